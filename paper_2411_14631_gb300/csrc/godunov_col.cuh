@@ -78,10 +78,10 @@ __device__ __forceinline__ void col_solve(const R WL[NV], const R WR[NV], const 
             flux_normal(W0, pr.gamma, Fn, U0);
         } else {
             set_error(status, e);
-            hllc(WL, WR, pr.gamma, Fn);
+            hllc(WL, WR, pr, Fn);
         }
     } else {
-        hllc(WL, WR, pr.gamma, Fn);
+        hllc(WL, WR, pr, Fn);
     }
 }
 
@@ -128,8 +128,7 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
     auto qx = [](int ix, int iy) { return (ix ^ (((iy >> 2) & 1) << 2)) + FX * iy; };
     const TreeView &tv = a.tv;
     const int tid = threadIdx.x, nt = blockDim.x;
-    Prm<R> pr;
-    pr.gamma = to_work<R>(a.gamma); pr.rho_floor = to_work<R>(a.rho_floor); pr.p_floor = to_work<R>(a.p_floor);
+    Prm<R> pr = make_prm<R>(a.gamma, a.rho_floor, a.p_floor);
     const R cflR = to_work<R>(a.cfl);
     const bool batch = a.n_inst > 0;
     const bool per[3] = {tv.bc[0] == AMR_BC_PERIODIC, tv.bc[2] == AMR_BC_PERIODIC, tv.bc[4] == AMR_BC_PERIODIC};

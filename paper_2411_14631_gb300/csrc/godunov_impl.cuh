@@ -182,6 +182,7 @@ __device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsig
 template <int D> __host__ __device__ constexpr int threads_for() { return D == 1 ? 128 : 512; }
 template <typename R, int D, int RS> constexpr int min_ctas_for()
 {
+    if (D == 1 && sizeof(R) == 8 && RS == AMR_RIEMANN_HLLC) return 3;
     return (D == 1 && sizeof(R) == 4 && RS != AMR_RIEMANN_MLP) ? 8 : 1;
 }
 
@@ -278,10 +279,10 @@ __device__ __forceinline__ void face_flux(Smem<R, D, RS> &sm, R (*sF)[NV][Geo<D>
             flux_normal(W0, pr.gamma, Fn, U0);
         } else {
             set_error(status, e);
-            hllc(WL, WR, pr.gamma, Fn);
+            hllc(WL, WR, pr, Fn);
         }
     } else {
-        hllc(WL, WR, pr.gamma, Fn);
+        hllc(WL, WR, pr, Fn);
     }
     sF[DIR][0][r0] = Fn[0];
     sF[DIR][N0][r0] = Fn[1];
@@ -366,7 +367,7 @@ __device__ __forceinline__ void mlp_faces(Smem<R, D, RS> &sm, R (*sF)[NV][Geo<D>
                 flux_normal(W0, g, Fn, U0);
             } else {
                 if (valid) set_error(a.status, e);
-                hllc(WL, WR, g, Fn);
+                hllc(WL, WR, pr, Fn);
             }
         }
         // accepted (seeded) faces and fallbacks (cold starts)
@@ -396,8 +397,7 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
     static_assert(3 * NV * G::NF <= NV * G::NC, "flux buffer must fit in the stencil buffer");
     const TreeView &tv = a.tv;
     const int tid = threadIdx.x;
-    Prm<R> pr;
-    pr.gamma = to_work<R>(a.gamma); pr.rho_floor = to_work<R>(a.rho_floor); pr.p_floor = to_work<R>(a.p_floor);
+    Prm<R> pr = make_prm<R>(a.gamma, a.rho_floor, a.p_floor);
     pr.limiter = a.limiter;
     const R cflR = to_work<R>(a.cfl);
 
@@ -732,8 +732,7 @@ static amr_status launch(const GArgs &a, int64_t ntile, cudaStream_t st)
     // 227 KB per CTA at most; the FP32 depth-1 update keeps eight CTAs in an SM's 228 KB
     // (each with its 1 KB reserved by the system)
     static_assert(sizeof(Smem<R, D, RS>) <= 227 * 1024, "tile shared memory");
-    static_assert(min_ctas_for<R, D, RS>() == 1 || (sizeof(Smem<R, D, RS>) + 1024) * 8 <= 228 * 1024,
-                  "eight depth-1 CTAs per SM");
+    static_assert((sizeof(Smem<R, D, RS>) + 1024) * min_ctas_for<R, D, RS>() <= 228 * 1024, "depth-1 CTAs per SM");
     const size_t bytes = sizeof(Smem<R, D, RS>);
     auto kern = k_godunov<R, D, RS>;
     AMR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));

@@ -5,6 +5,7 @@
 // solver (Ch. 4: pressure function, Newton from the PVRS guess, sampling at x/t = 0).
 #pragma once
 #include "common.cuh"
+#include "fp64_math.cuh"
 
 namespace amr {
 
@@ -86,6 +87,25 @@ template <typename R> struct Prm {
     int limiter = AMR_LIMITER_MINMOD;   // slopes of the reconstruction
 };
 
+// FP64: with 1/(gamma - 1) as the sum of two doubles, so that p/(gamma - 1) takes two
+// operations (within 0.5 ulp and the low part's rounding)
+template <> struct Prm<double> {
+    double gamma, rho_floor, p_floor;
+    double igm1, igm1_lo;
+    int limiter = AMR_LIMITER_MINMOD;
+};
+
+template <typename R> __device__ __forceinline__ Prm<R> make_prm(double gamma, double rho_floor, double p_floor)
+{
+    Prm<R> p;
+    p.gamma = to_work<R>(gamma); p.rho_floor = to_work<R>(rho_floor); p.p_floor = to_work<R>(p_floor);
+    if constexpr (sizeof(R) == 8) {
+        p.igm1 = recip(p.gamma - 1.0);
+        p.igm1_lo = __dmul_rn(__fma_rn(-(p.gamma - 1.0), p.igm1, 1.0), p.igm1);
+    }
+    return p;
+}
+
 // MinMod: zero when the differences disagree in sign (or one is zero), else the one of
 // smaller magnitude.  Written as the median of (0, a, b), four min/max operations: for
 // finite a, b the same value as the textbook branch (a zero result may carry either sign)
@@ -93,8 +113,11 @@ template <typename R> __device__ __forceinline__ R minmod(R a, R b)
 {
     return fmax(fmin(a, b), fmin(fmax(a, b), R(0)));
 }
+template <> __device__ __forceinline__ double minmod<double>(double a, double b) { return minmod64(a, b); }
 
+// a floored at b > 0 (b also when a is NaN)
 template <typename R> __device__ __forceinline__ R rmax(R a, R b) { return a > b ? a : b; }
+template <> __device__ __forceinline__ double rmax<double>(double a, double b) { return floor_at(a, b); }
 
 // Monotonized central limiter (van Leer 1977): zero when the differences disagree in
 // sign, else the central difference (a+b)/2 limited to twice either difference
@@ -114,6 +137,14 @@ template <typename R> __device__ __forceinline__ R slope(const Prm<R> &p, R a, R
 template <typename R>
 __device__ __forceinline__ void cons_to_prim_w(const R U[NV], const Prm<R> &p, R W[NV])
 {
+    if constexpr (sizeof(R) == 8) {
+        // twice the kinetic energy as momentum times velocity: 11 FP64 operations in all
+        const double rho = rmax(U[0], p.rho_floor), ir = recip(rho);
+        W[0] = rho; W[1] = mulr(U[1], ir); W[2] = mulr(U[2], ir); W[3] = mulr(U[3], ir);
+        const double k2 = mulr(rho, sq3(W[1], W[2], W[3]));
+        W[4] = rmax(mulr(p.gamma - 1.0, fmar(-0.5, k2, U[4])), p.p_floor);
+        return;
+    }
     const R rho = rmax(U[0], p.rho_floor), irho = R(1) / rho;
     const R u = mulr(U[1], irho), v = mulr(U[2], irho), w = mulr(U[3], irho);
     const R ek = mulr(mulr(R(0.5), rho), sq3(u, v, w));
@@ -147,11 +178,49 @@ __device__ __forceinline__ void flux_normal(const R W[NV], R g, R F[NV], R U[NV]
     U[0] = rho; U[1] = ru; U[2] = mulr(rho, v); U[3] = mulr(rho, w); U[4] = E;
 }
 
-// HLLC flux (Toro, Spruce & Speares 1994); the side used is chosen before computing,
-// so every face does one star state (no divergent branches, no register-array pointers).
-template <typename R>
-__device__ __forceinline__ void hllc(const R WL[NV], const R WR[NV], R g, R F[NV])
+// HLLC flux, FP64: about 60 operations on the FP64 pipe.  The star flux is written with the
+// star region's mass flux and pressure (Toro 2009, Sec. 10.4: p* = p_K + m (S* - u_K), m =
+// rho_K (S_K - u_K); F* = (rho* S*, rho* S*^2 + p*, rho* S* v_K, rho* S* w_K, S* (E* + p*))),
+// equal to F_K + S_K (U*_K - U_K) in exact arithmetic with 18 operations fewer.
+__device__ __forceinline__ void hllc(const double WL[NV], const double WR[NV], const Prm<double> &pr, double F[NV])
 {
+    const double g = pr.gamma;
+    const double rL = WL[0], uL = WL[1], pL = WL[4];
+    const double rR = WR[0], uR = WR[1], pR = WR[4];
+    const double cL = sqrt_quot(mulr(g, pL), rL), cR = sqrt_quot(mulr(g, pR), rR);
+    const double SL = fmin(uL - cL, uR - cR);
+    const double SR = fmax(uL + cL, uR + cR);
+    const double qL = SL - uL, qR = SR - uR;
+    const double mL = mulr(rL, qL), mR = mulr(rR, qR);   // mass fluxes through the outer waves
+    const double Ss = divide(fmar(-uR, mR, fmar(uL, mL, pR - pL)), mL - mR);
+    const bool supL = ge0(SL), pos = ge0(Ss), left = supL || pos;
+    const bool star = !supL && (pos || gt0(SR));
+    const double r = left ? rL : rR, u = left ? uL : uR, v = left ? WL[2] : WR[2], w = left ? WL[3] : WR[3];
+    const double p = left ? pL : pR;
+    const double E = fmar(0.5, mulr(r, sq3(u, v, w)), fmar(p, pr.igm1, mulr(p, pr.igm1_lo)));
+    if (star) {
+        const double m = left ? mL : mR;
+        const double d = recip((left ? SL : SR) - Ss);
+        const double ps = fmar(m, Ss - u, p);
+        const double Es = mulr(d, fmar(ps, Ss, fmar(-p, u, mulr(left ? qL : qR, E))));
+        F[0] = mulr(mulr(m, d), Ss);
+        F[1] = fmar(F[0], Ss, ps);
+        F[4] = mulr(Ss, Es + ps);
+    } else {
+        F[0] = mulr(r, u);
+        F[1] = fmar(F[0], u, p);
+        F[4] = mulr(u, E + p);
+    }
+    F[2] = mulr(F[0], v);
+    F[3] = mulr(F[0], w);
+}
+
+// HLLC flux, FP32 (Toro, Spruce & Speares 1994); the side used is chosen before computing,
+// so every face does one star state (no divergent branches, no register-array pointers).
+__device__ __forceinline__ void hllc(const float WL[NV], const float WR[NV], const Prm<float> &pr, float F[NV])
+{
+    using R = float;
+    const R g = pr.gamma;
     const R rL = WL[0], uL = WL[1], pL = WL[4];
     const R rR = WR[0], uR = WR[1], pR = WR[4];
     const R cL = sqrt(mulr(g, pL) / rL), cR = sqrt(mulr(g, pR) / rR);
@@ -302,6 +371,17 @@ template <typename R>
 __device__ __forceinline__ void muscl_predict(const R Wc[NV], const R Dl[3][NV], R hl, R gamma, R Wt[NV])
 {
     const R rr = Wc[0], u = Wc[1], vv = Wc[2], w = Wc[3], pp = Wc[4];
+    if constexpr (sizeof(R) == 8) {
+        // FP64: the velocity divergence formed once, 31 operations
+        const double div = (Dl[0][1] + Dl[1][2]) + Dl[2][3], ir = recip(rr);
+        auto adv = [&](int k) { return fmar(w, Dl[2][k], fmar(vv, Dl[1][k], mulr(u, Dl[0][k]))); };
+        Wt[0] = fmar(-hl, fmar(rr, div, adv(0)), rr);
+        Wt[1] = fmar(-hl, fmar(Dl[0][4], ir, adv(1)), u);
+        Wt[2] = fmar(-hl, fmar(Dl[1][4], ir, adv(2)), vv);
+        Wt[3] = fmar(-hl, fmar(Dl[2][4], ir, adv(3)), w);
+        Wt[4] = fmar(-hl, fmar(mulr(gamma, pp), div, adv(4)), pp);
+        return;
+    }
     R s = fmar(rr, Dl[2][3], fmar(w, Dl[2][0], fmar(rr, Dl[1][2], fmar(vv, Dl[1][0], fmar(rr, Dl[0][1],
                                                                                         mulr(u, Dl[0][0]))))));
     Wt[0] = fmar(-hl, s, rr);
@@ -339,9 +419,12 @@ __device__ __forceinline__ double cfl_candidate(const double U[NV], const Prm<R>
 {
     R W[NV];
     cons_to_prim(U, p, W);
+    if constexpr (sizeof(R) == 8) {
+        const double c = sqrt_quot(mulr(p.gamma, W[4]), W[0]);
+        return cfl * divide(dx, fmar(3.0, c, (fabs(W[1]) + fabs(W[2])) + fabs(W[3])));
+    }
     const R cs = sqrt(p.gamma * W[4] / W[0]);
     const R sig = (fabs(W[1]) + cs) + (fabs(W[2]) + cs) + (fabs(W[3]) + cs);
-    if (sizeof(R) == 8) return double(cfl) * (double(dx) / double(sig));
     // FP32: scaled down by (1 - 2^-16) so that it never exceeds the FP64 value
     return to_state(float(cfl) * (float(dx) / float(sig)) * 0.9999847412109375f);
 }

@@ -38,8 +38,7 @@ __global__ void k_courant(TreeView tv, int64_t cell0, const double *__restrict__
         double U[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) U[v] = u[v * tv.ncell + cell];
-        Prm<R> p;
-        p.gamma = to_work<R>(gamma); p.rho_floor = to_work<R>(rf); p.p_floor = to_work<R>(pf);
+        const Prm<R> p = make_prm<R>(gamma, rf, pf);
         const int l = tv.lvl[cell >> 3];
         cand = cfl_candidate<R>(U, p, to_work<R>(cfl), to_work<R>(pow2(-l)));
         if (lscale >= 0) cand = scale_pow2(cand, l - lscale);
@@ -80,8 +79,7 @@ __global__ void k_courant_batch(TreeView tv, const double *__restrict__ u, doubl
         double U[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) U[v] = u[v * tv.ncell + cell];
-        Prm<R> p;
-        p.gamma = to_work<R>(gamma); p.rho_floor = to_work<R>(rf); p.p_floor = to_work<R>(pf);
+        const Prm<R> p = make_prm<R>(gamma, rf, pf);
         cand = cfl_candidate<R>(U, p, to_work<R>(cfl), to_work<R>(tv.inst_dx[b]));
     }
     b = __shfl_sync(0xffffffffu, b, 0);
@@ -144,8 +142,7 @@ __device__ __forceinline__ double reflux_cell(const TreeView &tv, int level, int
 #pragma unroll
             for (int v = 0; v < NV; ++v) u[v * tv.ncell + cell] = U[v];
             if (want_dt) {
-                Prm<R> p;
-                p.gamma = to_work<R>(gamma); p.rho_floor = to_work<R>(rf); p.p_floor = to_work<R>(pf);
+                const Prm<R> p = make_prm<R>(gamma, rf, pf);
                 cand = cfl_candidate<R>(U, p, to_work<R>(cfl), to_work<R>(pow2(-level)));
             }
         }
@@ -275,8 +272,7 @@ __global__ void k_cons_to_prim(int64_t ncell, const double *__restrict__ u, doub
     double U[NV], W[NV];
 #pragma unroll
     for (int v = 0; v < NV; ++v) U[v] = u[v * ncell + i];
-    Prm<double> p;
-    p.gamma = gamma; p.rho_floor = rf; p.p_floor = pf;
+    const Prm<double> p = make_prm<double>(gamma, rf, pf);
     cons_to_prim(U, p, W);
 #pragma unroll
     for (int v = 0; v < NV; ++v) w[v * ncell + i] = W[v];
