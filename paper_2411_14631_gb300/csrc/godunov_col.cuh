@@ -50,18 +50,69 @@ struct ColArgs {
     // batch mode (n_inst > 0): per-box work offsets, octs lexicographic per box
     int32_t n_inst;
     const int64_t *inst_col_off, *inst_oct_off;
-    int64_t work;
+    // the z planes of every column, column after column (box after box): CTA i takes planes
+    // [i share, (i + 1) share), a segment per column it meets; with zc > 0 no segment is
+    // longer than zc and each CTA takes one (share = zc, columns padded to multiples of zc)
+    int64_t planes, share;
+    int zc;
     int32_t finer;          // the level has refined cells (finer levels exist)
     int level;
     int64_t n;              // cells per dimension
-    int zc;                 // segment length in cells (power of two, divides n)
     const double *u_old;
     double *u_new;
+    // u_old and u_new by variable: as kernel parameters they are operands of the address
+    // arithmetic, and take no registers
+    const double *uo[NV];
+    double *un[NV];
     const double *dt;
     double *dt_next;
     double gamma, rho_floor, p_floor, cfl;
     int32_t *status;
+
+    void scheme(const hydro_params *p)
+    {
+        gamma = p->gamma; rho_floor = p->rho_floor; p_floor = p->p_floor; cfl = p->cfl;
+        status = p->d_status;
+    }
+    void state(const amr_tree *t, const double *u0, double *u1)
+    {
+        u_old = u0;
+        u_new = u1;
+        for (int v = 0; v < NV; ++v) {
+            uo[v] = u0 + int64_t(v) * 8 * t->noct;
+            un[v] = u1 + int64_t(v) * 8 * t->noct;
+        }
+    }
 };
+
+// Even share of z planes per CTA.  A segment of s planes costs about s + extra plane steps
+// (its first planes are gathered and predicted without an update), a CTA meets at most
+// 1 + ceil((share - 2) / n) columns, and `slots` CTAs are resident: one wave of equal shares
+// keeps every SM busy to the end.  Segments of a fixed length in whole waves left up to a
+// sixth of the slots idle in the last wave and paid `extra` more often.
+inline int64_t even_share(int64_t planes, int64_t slots)
+{
+    int64_t s = (planes + slots - 1) / slots;
+    s += s & 1;
+    return s < 2 ? 2 : s;
+}
+
+// The next segment of a CTA that is at plane g (end: the end of its planes): the column of
+// height n it lies in (counted from plane `first` of this level or box) and [z0, z1) of it.
+struct ColSeg {
+    int col, z0, z1;
+};
+__device__ __forceinline__ ColSeg next_segment(int64_t first, int64_t g, int64_t end, int n, int zc)
+{
+    ColSeg s;
+    const int pitch = zc > 0 ? (n + zc - 1) / zc * zc : n;   // planes a column takes of the range
+    const int64_t r = g - first;
+    s.col = int(r / pitch);
+    s.z0 = int(r - int64_t(s.col) * pitch);
+    const int64_t z1 = s.z0 + (end - g);
+    s.z1 = int(z1 < n ? z1 : n);
+    return s;
+}
 
 // Riemann flux in the face-normal frame (HLLC, or the exact solver with HLLC fallback)
 template <typename R, int RS>
@@ -134,18 +185,11 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
     const bool per[3] = {tv.bc[0] == AMR_BC_PERIODIC, tv.bc[2] == AMR_BC_PERIODIC, tv.bc[4] == AMR_BC_PERIODIC};
     unsigned long long my_dt = ~0ull;
 
-    const double *uo[NV];
-    double *un[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        uo[v] = a.u_old + v * tv.ncell;
-        un[v] = a.u_new + v * tv.ncell;
-    }
-
-    for (int64_t b = blockIdx.x; b < a.work; b += gridDim.x) {
-        // geometry of this work item: the level (or the box), its column footprint and segment
+    const int64_t gend = min((int64_t(blockIdx.x) + 1) * a.share, a.planes);
+    for (int64_t g = blockIdx.x * a.share; g < gend;) {
+        // geometry of this segment: the level (or the box), its column footprint and z range
         int l = a.level;
-        int64_t n = a.n, wb = b;
+        int64_t n = a.n, first = 0;
         int32_t obase = 0;                        // batch: first oct of the box
         double dx, lam;
         double *dtn = a.dt_next;
@@ -153,10 +197,10 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
             int lo = 0, hi = a.n_inst - 1;
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
-                if (a.inst_col_off[mid] <= b) lo = mid; else hi = mid - 1;
+                if (a.inst_col_off[mid] * 16 <= g) lo = mid; else hi = mid - 1;
             }
             n = tv.inst_n[lo];
-            wb = b - a.inst_col_off[lo];
+            first = a.inst_col_off[lo] * 16;      // planes of 8 x 8 columns
             obase = int32_t(a.inst_oct_off[lo]);
             dx = tv.inst_dx[lo];
             lam = a.dt[lo] * double(n);
@@ -172,10 +216,12 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
         // cell coordinates, oct and cell ids fit in 32 bits (at most 2^12 cells per axis and
         // fewer than 2^27 octs)
         const int ni = int(n);
-        const int64_t nfx = n / FX, nfy = n / FY;
-        const int64_t fxy = wb % (nfx * nfy), seg = wb / (nfx * nfy);
-        const int X0 = int(fxy % nfx) * FX - 2, Y0 = int(fxy / nfx) * FY - 2;   // stencil index 0
-        const int z0 = int(seg) * a.zc;
+        const int nfx = ni / FX;
+        const ColSeg seg = next_segment(first, g, gend, ni, a.zc);
+        g += seg.z1 - seg.z0;
+        if (a.zc > 0) g = gend;                   // one segment per CTA
+        const int X0 = (seg.col % nfx) * FX - 2, Y0 = (seg.col / nfx) * FY - 2;   // stencil index 0
+        const int z0 = seg.z0, z1 = seg.z1;
         auto wrap = [&](int c, int axis) -> int {
             if (c >= 0 && c < ni) return c;
             if (per[axis]) return c < 0 ? c + ni : c - ni;   // within one period of the box
@@ -202,7 +248,7 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
                                 4 * (wrap(zp, 2) & 1);
             R Uw[NV], Wc[NV];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) Uw[v] = to_work<R>(uo[v][cid]);
+            for (int v = 0; v < NV; ++v) Uw[v] = to_work<R>(a.uo[v][cid]);
             cons_to_prim_w(Uw, pr, Wc);
 #pragma unroll
             for (int v = 0; v < NV; ++v) sm.W[zp & 3][v][i + SX * j] = Wc[v];
@@ -332,7 +378,7 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
             const int o = ((x + 2) >> 1) + (SX / 2) * ((y + 2) >> 1);
             const int32_t cid = sm.oct[(k >> 1) & 3][o] * 8 + (x & 1) + 2 * (y & 1) + 4 * dz;
 #pragma unroll
-            for (int v = 0; v < NV; ++v) Uo[v] = uo[v][cid];
+            for (int v = 0; v < NV; ++v) Uo[v] = a.uo[v][cid];
             return cid;
         };
         auto update = [&](int k, int q, const double Uo[NV], int32_t cid) {
@@ -370,7 +416,7 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
             for (int v = 0; v < NV; ++v) {
                 if (sizeof(R) == 8) Un[v] = Uo[v] + lam * to_state(dU[v]);
                 else Un[v] = Uo[v] + to_state(lamR * dU[v]);
-                un[v][cid] = Un[v];
+                a.un[v][cid] = Un[v];
                 sm.U[ub][uc][uo8 * NV + v] = Un[v];
             }
             if (!state_finite<R>(Un)) set_error(a.status, AMR_ENONPHYSICAL);
@@ -412,8 +458,8 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
         // per slab k: {update of slab k, gather of the layer slab k+2 needs, restriction of
         // slab k-2} share one phase, then the predictions and faces of slab k+2
         static_assert(NU <= 256, "one update item per thread of a 256-thread CTA");
-        for (int k = z0; k < z0 + a.zc; k += 2) {
-            const bool more = k + 2 < z0 + a.zc;
+        for (int k = z0; k < z1; k += 2) {
+            const bool more = k + 2 < z1;
             const int nwork = NU + (more ? NG : 0) + (k > z0 ? NR : 0);
             // a thread with an update item loads its old state first, so that the load
             // latency overlaps its gather or restriction item; the update follows them
@@ -436,7 +482,7 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
             // the oct table of layer k/2+3 (slot of the dead layer k/2-1), which the gather of
             // slab k+2 and the update of slab k+6 read, is filled beside the predictions; the
             // layer's state rows are prefetched into L2 beside the faces
-            const bool ahead = k + 4 < z0 + a.zc;
+            const bool ahead = k + 4 < z1;
             predict2(k + 3, ahead, k / 2 + 3);
             __syncthreads();
             slab_faces(k + 2, ahead, k / 2 + 3);
@@ -444,7 +490,7 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
         }
         // the last slab's restriction
         if (!batch)
-            for (int w = tid; w < NR; w += nt) restrict_one(z0 + a.zc - 2, w);
+            for (int w = tid; w < NR; w += nt) restrict_one(z1 - 2, w);
         if (batch && dtn) {
             // boxes have their own time steps: reduce this work item's candidates now
             for (int off = 16; off > 0; off >>= 1) my_dt = min(my_dt, __shfl_xor_sync(0xffffffffu, my_dt, off));
@@ -459,6 +505,16 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
     }
 }
 
+// CTAs of a kernel that are resident on the GPU at once
+template <typename K> inline int64_t resident_ctas(K kern, int threads, size_t smem)
+{
+    int dev = 0, nsm = 152, per_sm = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
+        per_sm = 1;
+    return int64_t(per_sm) * nsm;
+}
+
 template <typename R, int RS>
 amr_status launch_col(const amr_tree *t, const hydro_params *p, const double *u_old, double *u_new, const double *dt,
                       double *dt_next, cudaStream_t st)
@@ -471,32 +527,27 @@ amr_status launch_col(const amr_tree *t, const hydro_params *p, const double *u_
     a.inst_col_off = t->inst_col_off;
     a.inst_oct_off = t->inst_oct_off;
     a.finer = t->n_inst == 0 && t->grid_level < t->levelmax;
+    a.zc = 0;
     if (t->n_inst > 0) {
         a.level = 0;
         a.n = 0;
-        a.zc = 16;
-        a.work = t->col_work;
+        a.planes = t->col_work * 16;
     } else {
         a.level = t->grid_level;
         a.n = int64_t(1) << t->grid_level;
-        // longest segment (at most 64 cells, fewer prologue planes per cell) that still
-        // gives two waves of four CTAs per SM
-        int dev = 0, nsm = 152;
-        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        a.zc = a.n < 64 ? int(a.n) : 64;
-        while (a.zc > 16 && (a.n / FX) * (a.n / FY) * (a.n / a.zc) < int64_t(8) * nsm) a.zc /= 2;
+        a.planes = (a.n / FX) * (a.n / FY) * a.n;
         const int want = p->col_seg;
         if (want >= 2 && want <= a.n && (want & (want - 1)) == 0) a.zc = want;
-        a.work = (a.n / FX) * (a.n / FY) * (a.n / a.zc);
     }
-    a.u_old = u_old; a.u_new = u_new; a.dt = dt; a.dt_next = dt_next;
-    a.gamma = p->gamma; a.rho_floor = p->rho_floor; a.p_floor = p->p_floor; a.cfl = p->cfl;
-    a.status = p->d_status;
+    a.state(t, u_old, u_new);
+    a.dt = dt; a.dt_next = dt_next;
+    a.scheme(p);
     const bool finer = a.finer != 0;
     const size_t bytes = finer ? sizeof(ColSmem<R, FX, FY, true>) : sizeof(ColSmem<R, FX, FY, false>);
     auto kern = finer ? k_godunov_col<R, RS, FX, FY, true> : k_godunov_col<R, RS, FX, FY, false>;
     AMR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
-    kern<<<unsigned(a.work < 1048576 ? a.work : 1048576), 256, bytes, st>>>(a);
+    a.share = a.zc > 0 ? a.zc : even_share(a.planes, resident_ctas(kern, 256, bytes));
+    kern<<<unsigned((a.planes + a.share - 1) / a.share), 256, bytes, st>>>(a);
     AMR_CUDA_TRY(cudaGetLastError());
     return AMR_OK;
 }

@@ -33,6 +33,17 @@ __device__ __forceinline__ float d2f_bits(double x)
     return __uint_as_float(m | (hi & 0x80000000u));
 }
 
+// The same where denormal values are flushed by their use (the FP32 kernels), both ends of the
+// range clamped by one instruction: 6 integer operations instead of 8.  Where d2f_bits gives
+// a zero for |x| < 2^-126 this gives a denormal (or, rounded up to it, 2^-126).
+__device__ __forceinline__ float d2f_ftz(double x)
+{
+    const unsigned hi = unsigned(__double2hiint(x)), lo = unsigned(__double2loint(x));
+    const unsigned r = unsigned(__viaddmin_s32_relu(int(hi & 0x7FFFFFFFu), -(896 << 20), 255 << 20));
+    const unsigned long long b = ((static_cast<unsigned long long>(r) << 32) | lo) + (1ull << 28);
+    return __uint_as_float(unsigned(b >> 29) | (hi & 0x80000000u));
+}
+
 __device__ __forceinline__ double f2d_bits(float f)
 {
     const unsigned b = __float_as_uint(f), ab = b & 0x7FFFFFFFu;
@@ -42,6 +53,17 @@ __device__ __forceinline__ double f2d_bits(float f)
     const unsigned hi = z ? 0u : (ab >> 3) + bias;
     const unsigned lo = z ? 0u : ab << 29;
     return __hiloint2double(int(hi | (b & 0x80000000u)), int(lo));
+}
+
+// x + f, f zero or normal, infinite or NaN (the FP32 kernels flush denormals): f's bits shifted
+// into a double of 2^-896 times its value (exponent field kept), scaled back exactly inside
+// the multiply-add; Inf and NaN get the double's exponent field.  The same as x + f2d_bits(f).
+__device__ __forceinline__ double add_f32(double x, float f)
+{
+    const int b = __float_as_int(f);
+    int hi = (b >> 3) & int(0x8FFFFFFFu);
+    if (!(fabsf(f) <= 3.402823466e38f)) hi |= 0x7FF00000;
+    return __fma_rn(__hiloint2double(hi, b << 29), __longlong_as_double((1023ll + 896ll) << 52), x);
 }
 
 // whether the five values of an FP64 state are finite in the working precision R: for
@@ -58,14 +80,14 @@ template <> __device__ __forceinline__ bool state_finite<double>(const double U[
 }
 template <> __device__ __forceinline__ bool state_finite<float>(const double U[5])
 {
-    const float s = (d2f_bits(U[0]) + d2f_bits(U[1])) + (d2f_bits(U[2]) + d2f_bits(U[3])) + d2f_bits(U[4]);
+    const float s = (d2f_ftz(U[0]) + d2f_ftz(U[1])) + (d2f_ftz(U[2]) + d2f_ftz(U[3])) + d2f_ftz(U[4]);
     return fabsf(s) <= 3.402823466e38f;
 }
 
 // working-precision view of an FP64 state value, and back
 template <typename R> __device__ __forceinline__ R to_work(double x);
 template <> __device__ __forceinline__ double to_work<double>(double x) { return x; }
-template <> __device__ __forceinline__ float to_work<float>(double x) { return d2f_bits(x); }
+template <> __device__ __forceinline__ float to_work<float>(double x) { return d2f_ftz(x); }
 __device__ __forceinline__ double to_state(double x) { return x; }
 __device__ __forceinline__ double to_state(float x) { return f2d_bits(x); }
 
@@ -236,21 +258,17 @@ __device__ __forceinline__ void hllc(const float WL[NV], const float WR[NV], con
     const R SK = left ? SL : SR;
     R FK[NV], UK[NV];
     flux_normal(WK, g, FK, UK);
-    if (star) {
-        // U*_K = f [1, S*, v_K, w_K, E_K/rho_K + (S* - u_K)(S* + p_K/(rho_K (S_K - u_K)))],
-        // f = rho_K (S_K - u_K) / (S_K - S*); with d = 1/(S_K - S*) the energy component is
-        // d ((S_K - u_K) E_K + (S* - u_K) p_K) + f (S* - u_K) S*, one division in all
-        const R rK = WK[0], uK = WK[1], pK = WK[4];
-        const R d = R(1) / (SK - Ss);
-        const R f = mulr(mulr(rK, SK - uK), d);
-        const R Us[NV] = {f, mulr(f, Ss), mulr(f, WK[2]), mulr(f, WK[3]),
-                          fmar(mulr(f, Ss - uK), Ss, mulr(d, fmar(Ss - uK, pK, mulr(SK - uK, UK[4]))))};
+    // U*_K = f [1, S*, v_K, w_K, E_K/rho_K + (S* - u_K)(S* + p_K/(rho_K (S_K - u_K)))],
+    // f = rho_K (S_K - u_K) / (S_K - S*); with d = 1/(S_K - S*) the energy component is
+    // d ((S_K - u_K) E_K + (S* - u_K) p_K) + f (S* - u_K) S*, one division in all
+    const R rK = WK[0], uK = WK[1], pK = WK[4];
+    const R d = R(1) / (SK - Ss);
+    const R f = mulr(mulr(rK, SK - uK), d);
+    const R Us[NV] = {f, mulr(f, Ss), mulr(f, WK[2]), mulr(f, WK[3]),
+                      fmar(mulr(f, Ss - uK), Ss, mulr(d, fmar(Ss - uK, pK, mulr(SK - uK, UK[4]))))};
+    // formed on both sides of the choice: without a branch the solves of different faces overlap
 #pragma unroll
-        for (int v = 0; v < NV; ++v) F[v] = fmar(SK, Us[v] - UK[v], FK[v]);
-    } else {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) F[v] = FK[v];
-    }
+    for (int v = 0; v < NV; ++v) F[v] = star ? fmar(SK, Us[v] - UK[v], FK[v]) : FK[v];
 }
 
 // Toro Eq. 4.6-4.7: one side's contribution to the pressure function and derivative
@@ -414,6 +432,22 @@ __device__ __forceinline__ void face_state(const R Wt[NV], const R DlD[NV], R ha
 
 // dt candidate of one cell: cfl * dx / sum_d (|u_d| + c), from the FP64 state; p, cfl and
 // dx already in the working precision
+// FP32, in two parts: the candidate of a cell falls with its signal speed sum_d (|u_d| + c)
+// (rcp.approx.ftz.f32, which the division is made of, falls monotonically over all normal
+// floats: checked value by value), so the smallest candidate of cells of one size is that
+// of their largest signal speed.
+__device__ __forceinline__ float cfl_signal(const double U[NV], const Prm<float> &p)
+{
+    float W[NV];
+    cons_to_prim(U, p, W);
+    const float cs = sqrt(p.gamma * W[4] / W[0]);
+    return (fabs(W[1]) + cs) + (fabs(W[2]) + cs) + (fabs(W[3]) + cs);
+}
+__device__ __forceinline__ double cfl_step(float sig, float cfl, float dx)
+{
+    return to_state(cfl * (dx / sig) * 0.9999847412109375f);
+}
+
 template <typename R>
 __device__ __forceinline__ double cfl_candidate(const double U[NV], const Prm<R> &p, R cfl, R dx)
 {
