@@ -174,83 +174,73 @@ __global__ void k_reflux_list(TreeView tv, int level, const int32_t *__restrict_
     if (dt_next) min_to(dt_next, cand);
 }
 
-// Restriction of complete levels: one CTA per oct O of level L restricts the nlev levels
-// L + nlev - 1 .. L of O's subtree (nlev <= 3), the deepest from level L + nlev in global
-// memory, the others from the values it has just formed (kept in shared memory).  Every
-// cell is the mean of its eight children summed in cell order, as in k_reflux.  Valid
+// Restriction of complete levels: one CTA per oct O of level L and variable restricts the nlev
+// levels L + nlev - 1 .. L of O's subtree (nlev <= 3), the deepest from level L + nlev in
+// global memory, the others from the values it has just formed (kept in shared memory).
+// Every cell is the mean of its eight children summed in cell order, as in k_reflux.  Valid
 // where levels L .. L + nlev are complete (every cell of levels L .. L + nlev - 1 refined):
-// the levels below the deepest complete one.
+// the levels below the deepest complete one.  There the octs of a subtree are consecutive on
+// every level (they are sorted by Hilbert key, whose prefix is the father's), so all son
+// entries a CTA needs load at once instead of level after level.
+//
+// Bound: latency (one look-up, one read, nine FP64 operations per level) and, for the large
+// launches, reads at 64 bytes per (cell, variable).  A CTA for all five variables that
+// followed the son tables down took 16 us for the three top levels (its 26 k FP64 operations
+// alone take 6 us on one SM) and 38 us for levels 6-4 of a 256^3 box.
 __global__ void __launch_bounds__(256) k_restrict_complete(TreeView tv, int L, int nlev, double *u)
 {
-    __shared__ int32_t son1[8], son2[64], son3[512];   // son octs of O's cells, of theirs, ...
-    __shared__ double v2[NV][512], v1[NV][64];
+    __shared__ int32_t son1[8], son2[64];   // son octs of the cells of levels L and L + 1, from the subtree's first
+    __shared__ double v2[512], v1[64];
     const int t = threadIdx.x;
-    const int64_t O = tv.lvl_off[L] + blockIdx.x;
+    const int64_t o = blockIdx.x, O = tv.lvl_off[L] + o;
+    const int64_t b1 = tv.lvl_off[L + 1] + 8 * o, b2 = nlev > 1 ? tv.lvl_off[L + 2] + 64 * o : 0;
+    double *uv = u + blockIdx.y * tv.ncell;
     auto mean8 = [&](const double *c) {
         double acc = 0.0;
 #pragma unroll
         for (int q = 0; q < 8; ++q) acc += c[q];
         return 0.125 * acc;
     };
-    if (nlev >= 2 && t < 8) son1[t] = tv.son[O * 8 + t];
-    __syncthreads();
-    if (nlev == 3 && t < 64) son2[t] = tv.son[int64_t(son1[t >> 3]) * 8 + (t & 7)];
-    __syncthreads();
-    if (nlev == 3) {
-        for (int j = t; j < 512; j += blockDim.x) son3[j] = tv.son[int64_t(son2[j >> 3]) * 8 + (j & 7)];
-        __syncthreads();
-        // level L+2: the 512 cells of the 64 octs son2[], from their sons son3[] at level L+3
-#pragma unroll 2
-        for (int w = t; w < 512 * NV; w += blockDim.x) {
-            const int v = w >> 9, j = w & 511;
-            const double2 *src = reinterpret_cast<const double2 *>(u + v * tv.ncell + int64_t(son3[j]) * 8);
-            double c[8];
+    const bool vec = (reinterpret_cast<uintptr_t>(u) & 15) == 0;
+    auto mean_of = [&](int32_t oct) {
+        const double *src = uv + int64_t(oct) * 8;
+        double c[8];
+        if (vec) {
 #pragma unroll
             for (int h = 0; h < 4; ++h) {
-                const double2 q2 = src[h];
+                const double2 q2 = reinterpret_cast<const double2 *>(src)[h];
                 c[2 * h] = q2.x;
                 c[2 * h + 1] = q2.y;
             }
-            const double m = mean8(c);
-            u[v * tv.ncell + int64_t(son2[j >> 3]) * 8 + (j & 7)] = m;
-            v2[v][j] = m;
+        } else {
+#pragma unroll
+            for (int h = 0; h < 8; ++h) c[h] = src[h];
         }
-        __syncthreads();
+        return mean8(c);
+    };
+    if (nlev > 1 && t < 8) son1[t] = int32_t(tv.son[O * 8 + t] - b1);
+    if (nlev > 2 && t >= 32 && t < 96) son2[t - 32] = int32_t(tv.son[b1 * 8 + t - 32] - b2);
+    if (nlev == 3) {
+        // level L + 2: the 512 cells of 64 octs
+#pragma unroll
+        for (int j = t; j < 512; j += 256) {
+            const double m = mean_of(tv.son[b2 * 8 + j]);
+            uv[b2 * 8 + j] = m;
+            v2[j] = m;
+        }
     }
+    __syncthreads();
     if (nlev >= 2) {
-        // level L+1: the 64 cells of the 8 octs son1[]
-        for (int w = t; w < 64 * NV; w += blockDim.x) {
-            const int v = w >> 6, k = w & 63;
-            const int64_t cell = int64_t(son1[k >> 3]) * 8 + (k & 7);
-            double c[8];
-            if (nlev == 3) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q) c[q] = v2[v][k * 8 + q];
-            } else {
-                const int64_t s2 = tv.son[cell];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) c[q] = u[v * tv.ncell + s2 * 8 + q];
-            }
-            const double m = mean8(c);
-            u[v * tv.ncell + cell] = m;
-            v1[v][k] = m;
+        // level L + 1: the 64 cells of eight octs
+        if (t < 64) {
+            const double m = nlev == 3 ? mean8(v2 + son2[t] * 8) : mean_of(tv.son[b1 * 8 + t]);
+            uv[b1 * 8 + t] = m;
+            v1[t] = m;
         }
         __syncthreads();
     }
     // level L: O's eight cells
-    if (t < 8 * NV) {
-        const int v = t >> 3, c0 = t & 7;
-        double c[8];
-        if (nlev >= 2) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) c[q] = v1[v][c0 * 8 + q];
-        } else {
-            const int64_t s1 = tv.son[O * 8 + c0];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) c[q] = u[v * tv.ncell + s1 * 8 + q];
-        }
-        u[v * tv.ncell + O * 8 + c0] = mean8(c);
-    }
+    if (t < 8) uv[O * 8 + t] = nlev >= 2 ? mean8(v1 + son1[t] * 8) : mean_of(tv.son[O * 8 + t]);
 }
 
 __global__ void k_prim_to_cons(int64_t ncell, const double *__restrict__ w, double *u, double gamma)
@@ -343,7 +333,7 @@ static amr_status restrict_complete_launch(const amr_tree *t, int lo_end, double
         const int L = top - nlev + 1;
         const int64_t nb = t->lvl_off[L + 1] - t->lvl_off[L];
         if (nb > 0) {
-            k_restrict_complete<<<unsigned(nb), 256, 0, st>>>(tv, L, nlev, u);
+            k_restrict_complete<<<dim3(unsigned(nb), NV), 256, 0, st>>>(tv, L, nlev, u);
             AMR_CUDA_TRY(cudaGetLastError());
         }
         top = L - 1;
