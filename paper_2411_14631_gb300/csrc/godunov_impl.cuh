@@ -91,6 +91,21 @@ __device__ __forceinline__ int64_t coarse_neighbour(const TreeView &tv, int64_t 
     return so >= 0 ? int64_t(so) * 8 + cc : int64_t(N);
 }
 
+// the cells the interpolation of coarse leaf cell F reads beside it, below and above on each axis
+__device__ __forceinline__ void interp_cells(const TreeView &tv, int64_t F, int64_t nm[3], int64_t np[3])
+{
+    const int64_t oF = F >> 3;
+    const int cf = int(F & 7);
+    const int lc = tv.lvl[oF];
+    const int64_t X[3] = {2 * int64_t(tv.ix[oF]) + (cf & 1), 2 * int64_t(tv.iy[oF]) + ((cf >> 1) & 1),
+                          2 * int64_t(tv.iz[oF]) + ((cf >> 2) & 1)};
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        nm[d] = coarse_neighbour(tv, oF, X, lc, d, -1);
+        np[d] = coarse_neighbour(tv, oF, X, lc, d, +1);
+    }
+}
+
 // The interpolation of coarse leaf cell F to its children, on conserved variables in the
 // working precision R (FP64 values read from the state): its value uc and its MinMod
 // slopes m[d] = minmod(U_F - U_{F-e_d}, U_{F+e_d} - U_F) ...
@@ -98,17 +113,8 @@ template <typename R>
 __device__ __forceinline__ void interp_slopes(const TreeView &tv, const double *__restrict__ u, int64_t F,
                                               R uc[NV], R m[3][NV])
 {
-    const int64_t oF = F >> 3;
-    const int cf = int(F & 7);
-    const int lc = tv.lvl[oF];
-    const int64_t X[3] = {2 * int64_t(tv.ix[oF]) + (cf & 1), 2 * int64_t(tv.iy[oF]) + ((cf >> 1) & 1),
-                          2 * int64_t(tv.iz[oF]) + ((cf >> 2) & 1)};
     int64_t nm[3], np[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        nm[d] = coarse_neighbour(tv, oF, X, lc, d, -1);
-        np[d] = coarse_neighbour(tv, oF, X, lc, d, +1);
-    }
+    interp_cells(tv, F, nm, np);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         uc[v] = to_work<R>(u[v * tv.ncell + F]);

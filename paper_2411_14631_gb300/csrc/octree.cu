@@ -107,7 +107,9 @@ static amr_status check_geom(const amr_geom *g, int64_t n)
 }
 
 // ---- kernels --------------------------------------------------------------------
-__global__ void k_keys(const int32_t *__restrict__ lxyz, int64_t n, uint64_t *sk, int32_t *id, int32_t *err)
+// sort key: the level above the kb bits of the deepest level's Hilbert keys, so that the sort
+// passes over no bits that are always zero
+__global__ void k_keys(const int32_t *__restrict__ lxyz, int64_t n, int kb, uint64_t *sk, int32_t *id, int32_t *err)
 {
     const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
     if (i >= n) return;
@@ -118,22 +120,39 @@ __global__ void k_keys(const int32_t *__restrict__ lxyz, int64_t n, uint64_t *sk
         set_error(err, AMR_EINVAL);
         sk[i] = ~uint64_t(0);
     } else {
-        sk[i] = (uint64_t(l) << 58) | hilbert3(l - 1, x, y, z);
+        sk[i] = (uint64_t(l) << kb) | hilbert3(l - 1, x, y, z);
     }
     id[i] = int32_t(i);
 }
 
-// octs per level of a device oct list (checked against the counts the caller gave)
-__global__ void k_level_hist(const int32_t *__restrict__ lxyz, int64_t n, unsigned long long *hist)
+// octs per level of a device oct list (checked against the counts the caller gave): counted in
+// shared memory, a warp whose octs share a level with one addition, then one global addition
+// per block and level (a global addition per oct serialised on a handful of addresses: 307 us
+// for 0.43 M octs)
+__global__ void __launch_bounds__(256) k_level_hist(const int32_t *__restrict__ lxyz, int64_t n,
+                                                    unsigned long long *hist)
 {
-    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (i >= n) return;
-    const int l = lxyz[4 * i];
-    if (l >= 0 && l < AMR_MAXLEV + 2) atomicAdd(hist + l, 1ull);
+    __shared__ int cnt[AMR_MAXLEV + 2];
+    if (threadIdx.x < AMR_MAXLEV + 2) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t stride = int64_t(gridDim.x) * blockDim.x;
+    for (int64_t i0 = blockIdx.x * int64_t(blockDim.x); i0 < n; i0 += stride) {
+        const int64_t i = i0 + threadIdx.x;
+        const int l = i < n ? lxyz[4 * i] : -1;
+        const int l0 = __shfl_sync(0xffffffffu, l, 0);
+        const bool ok = l >= 0 && l < AMR_MAXLEV + 2;
+        if (__all_sync(0xffffffffu, l == l0)) {
+            if (ok && (threadIdx.x & 31) == 0) atomicAdd(cnt + l, 32);
+        } else if (ok) {
+            atomicAdd(cnt + l, 1);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < AMR_MAXLEV + 2 && cnt[threadIdx.x]) atomicAdd(hist + threadIdx.x, (unsigned long long)cnt[threadIdx.x]);
 }
 
 __global__ void k_scatter(const uint64_t *__restrict__ sk, const int32_t *__restrict__ id,
-                          const int32_t *__restrict__ lxyz, int64_t n, int32_t *lvl, int32_t *ix, int32_t *iy,
+                          const int32_t *__restrict__ lxyz, int64_t n, int kb, int32_t *lvl, int32_t *ix, int32_t *iy,
                           int32_t *iz, uint64_t *key, int32_t *err)
 {
     const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
@@ -143,7 +162,7 @@ __global__ void k_scatter(const uint64_t *__restrict__ sk, const int32_t *__rest
     ix[i] = lxyz[4 * s + 1];
     iy[i] = lxyz[4 * s + 2];
     iz[i] = lxyz[4 * s + 3];
-    key[i] = sk[i] & ((uint64_t(1) << 58) - 1);
+    key[i] = sk[i] & ((uint64_t(1) << kb) - 1);
     if (i > 0 && sk[i] == sk[i - 1]) set_error(err, AMR_EINVAL);   // duplicate oct
 }
 
@@ -164,52 +183,65 @@ __device__ int64_t cell_of(const BuildView &b, int l, int64_t X, int64_t Y, int6
 }
 
 // Tables by search (son, father, nbor, nb27, refmask) for the octs [0, o1): levels 1 and 2,
-// whose neighbours cannot come from a coarser oct's table (the root's has no wrap).
+// whose neighbours cannot come from a coarser oct's table (the root's has no wrap).  A warp
+// per oct and an entry per lane (nine octs in all: one thread per oct made 42 searches in a
+// row, 50 us).
 __global__ void k_tables(BuildView b, int64_t o1, int32_t *son, int32_t *father, int32_t *nbor, int32_t *nb27,
                          uint8_t *refmask, int32_t *err)
 {
-    const int64_t o = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    const int64_t o = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
+    const int k = threadIdx.x & 31;
     if (o >= o1) return;
     const int l = b.lvl[o];
     const int64_t x = b.ix[o], y = b.iy[o], z = b.iz[o];
-    uint32_t mask = 0;
-    for (int c = 0; c < 8; ++c) {
-        const int64_t s = find_oct(b.key, b.lvl_off, l + 1, 2 * x + (c & 1), 2 * y + ((c >> 1) & 1), 2 * z + ((c >> 2) & 1));
-        son[8 * o + c] = int32_t(s);
-        if (s >= 0) mask |= 1u << c;
+    int64_t s = -1;
+    if (k < 8) {
+        s = find_oct(b.key, b.lvl_off, l + 1, 2 * x + (k & 1), 2 * y + ((k >> 1) & 1), 2 * z + ((k >> 2) & 1));
+        son[8 * o + k] = int32_t(s);
     }
-    refmask[o] = uint8_t(mask);
-    if (l < b.levelmin && mask != 0xFFu) set_error(err, AMR_EINVAL);   // levels below levelmin have no leaves
+    const uint32_t mask = __ballot_sync(0xffffffffu, s >= 0) & 0xFFu;
+    if (k == 0) {
+        refmask[o] = uint8_t(mask);
+        if (l < b.levelmin && mask != 0xFFu) set_error(err, AMR_EINVAL);   // levels below levelmin have no leaves
+    }
     if (l == 1) {
-        father[o] = -1;
-        for (int k = 0; k < 6; ++k) nbor[6 * o + k] = -1;
-        for (int k = 0; k < 27; ++k) nb27[27 * o + k] = (k == 13) ? int32_t(o) : OUTSIDE;
+        if (k == 0) father[o] = -1;
+        if (k < 6) nbor[6 * o + k] = -1;
+        if (k < 27) nb27[27 * o + k] = (k == 13) ? int32_t(o) : OUTSIDE;
         return;
     }
-    const int64_t f = cell_of(b, l - 1, x, y, z);
-    if (f < 0) set_error(err, AMR_EINVAL);                             // oct without its father cell
-    father[o] = int32_t(f);
+    if (k == 0) {
+        const int64_t f = cell_of(b, l - 1, x, y, z);
+        if (f < 0) set_error(err, AMR_EINVAL);                             // oct without its father cell
+        father[o] = int32_t(f);
+    }
     const int64_t nf = int64_t(1) << (l - 1);
-    for (int k = 0; k < 6; ++k) {
+    if (k < 6) {
         int64_t P[3] = {x, y, z};
         P[k >> 1] += (k & 1) ? 1 : -1;
         int out = 0;
         for (int a = 0; a < 3; ++a) out |= bc_apply(b.bc, a, nf, P[a]);
-        if (out) { nbor[6 * o + k] = -1; continue; }
-        const int64_t cid = cell_of(b, l - 1, P[0], P[1], P[2]);
-        if (cid < 0) set_error(err, AMR_EUNBALANCED);
+        int64_t cid = -1;
+        if (!out) {
+            cid = cell_of(b, l - 1, P[0], P[1], P[2]);
+            if (cid < 0) set_error(err, AMR_EUNBALANCED);
+        }
         nbor[6 * o + k] = int32_t(cid);
     }
-    for (int k = 0; k < 27; ++k) {
-        const int dx = k % 3 - 1, dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
-        int64_t P[3] = {x + dx, y + dy, z + dz};
+    if (k < 27) {
+        int64_t P[3] = {x + k % 3 - 1, y + (k / 3) % 3 - 1, z + k / 9 - 1};
         int out = 0;
         for (int a = 0; a < 3; ++a) out |= bc_apply(b.bc, a, nf, P[a]);
-        if (out) { nb27[27 * o + k] = OUTSIDE; continue; }
-        const int64_t cid = cell_of(b, l - 1, P[0], P[1], P[2]);   // 2:1 rule: must exist
-        if (cid < 0) { set_error(err, AMR_EUNBALANCED); nb27[27 * o + k] = OUTSIDE; continue; }
-        const int64_t s = find_oct(b.key, b.lvl_off, l, P[0], P[1], P[2]);
-        nb27[27 * o + k] = s >= 0 ? int32_t(s) : int32_t(-1 - cid);
+        int32_t e = OUTSIDE;
+        if (!out) {
+            const int64_t cid = cell_of(b, l - 1, P[0], P[1], P[2]);   // 2:1 rule: must exist
+            if (cid < 0) set_error(err, AMR_EUNBALANCED);
+            else {
+                const int64_t so = find_oct(b.key, b.lvl_off, l, P[0], P[1], P[2]);
+                e = so >= 0 ? int32_t(so) : int32_t(-1 - cid);
+            }
+        }
+        nb27[27 * o + k] = e;
     }
 }
 
@@ -235,49 +267,46 @@ __global__ void k_father_son(BuildView b, int32_t *son, int32_t *father, int32_t
 // Tables of the level-l octs (l >= 3) from the tables of their fathers' octs: the level-(l-1)
 // cell next to an oct's father lies in the father oct or one of its 26 neighbours, and the
 // level-l neighbour oct is that cell's son.  Same entries as k_tables, without searching.
+// One thread per oct and neighbour: rows are written by consecutive threads.
 __global__ void k_tables_level(BuildView b, int l, const int32_t *__restrict__ son, const int32_t *__restrict__ father,
                                int32_t *nbor, int32_t *nb27, uint8_t *refmask, int32_t *err)
 {
-    const int64_t o = b.lvl_off[l] + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    const int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    const int64_t o = b.lvl_off[l] + i / 27;
+    const int k = int(i % 27);
     if (o >= b.lvl_off[l + 1]) return;
-    const int32_t x = b.ix[o], y = b.iy[o], z = b.iz[o];   // father cell coordinates (level l-1)
-    uint32_t mask = 0;
+    if (k == 13) {
+        uint32_t mask = 0;
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
-        if (son[8 * o + c] >= 0) mask |= 1u << c;
-    refmask[o] = uint8_t(mask);
-    if (l < b.levelmin && mask != 0xFFu) set_error(err, AMR_EINVAL);   // levels below levelmin have no leaves
-    const int32_t f = father[o];
-    if (f < 0) return;                                                 // reported by k_father_son
-    const int32_t *pn = nb27 + 27 * int64_t(f >> 3);                   // the father's oct (level l-1)
-    // level-(l-1) cell (X, Y, Z) next to the father: its oct among the father oct's 27
-    auto cell_near = [&](int32_t X, int32_t Y, int32_t Z, int32_t &cid) -> int {
-        const int k = ((X >> 1) - (x >> 1) + 1) + 3 * ((Y >> 1) - (y >> 1) + 1) + 9 * ((Z >> 1) - (z >> 1) + 1);
-        const int32_t po = pn[k];
-        if (po == OUTSIDE) return 1;                                   // beyond an outflow face
-        if (po < 0) return 2;                                          // missing: 2:1 rule broken
-        cid = po * 8 + (X & 1) + 2 * (Y & 1) + 4 * (Z & 1);
-        return 0;
-    };
-    for (int k = 0; k < 6; ++k) {
-        int32_t P[3] = {x, y, z};
-        P[k >> 1] += (k & 1) ? 1 : -1;
-        int32_t cid = -1;
-        const int r = cell_near(P[0], P[1], P[2], cid);
-        if (r == 2) set_error(err, AMR_EUNBALANCED);
-        nbor[6 * o + k] = r == 0 ? cid : -1;
+        for (int c = 0; c < 8; ++c)
+            if (son[8 * o + c] >= 0) mask |= 1u << c;
+        refmask[o] = uint8_t(mask);
+        if (l < b.levelmin && mask != 0xFFu) set_error(err, AMR_EINVAL);   // levels below levelmin have no leaves
     }
-    for (int k = 0; k < 27; ++k) {
-        const int dx = k % 3 - 1, dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
-        int32_t cid = -1;
-        const int r = cell_near(x + dx, y + dy, z + dz, cid);
-        if (r != 0) {
-            if (r == 2) set_error(err, AMR_EUNBALANCED);
-            nb27[27 * o + k] = OUTSIDE;
-            continue;
-        }
+    const int32_t f = father[o];
+    if (f < 0) {                                                       // reported by k_father_son
+        nb27[27 * o + k] = OUTSIDE;
+        if (k < 6) nbor[6 * o + k] = -1;
+        return;
+    }
+    const int32_t x = b.ix[o], y = b.iy[o], z = b.iz[o];   // father cell coordinates (level l-1)
+    // level-(l-1) cell (X, Y, Z) next to the father: its oct among the father oct's 27
+    const int32_t X = x + k % 3 - 1, Y = y + (k / 3) % 3 - 1, Z = z + k / 9 - 1;
+    const int kp = ((X >> 1) - (x >> 1) + 1) + 3 * ((Y >> 1) - (y >> 1) + 1) + 9 * ((Z >> 1) - (z >> 1) + 1);
+    const int32_t po = nb27[27 * int64_t(f >> 3) + kp];                // an oct of level l-1
+    int32_t cid = -1, e = OUTSIDE;                                     // beyond an outflow face
+    if (po >= 0) {
+        cid = po * 8 + (X & 1) + 2 * (Y & 1) + 4 * (Z & 1);
         const int32_t sn = son[cid];
-        nb27[27 * o + k] = sn >= 0 ? sn : -1 - cid;
+        e = sn >= 0 ? sn : -1 - cid;
+    } else if (po != OUTSIDE) {
+        set_error(err, AMR_EUNBALANCED);                               // missing: 2:1 rule broken
+    }
+    nb27[27 * o + k] = e;
+    const int dx = k % 3 - 1, dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
+    if (dx * dx + dy * dy + dz * dz == 1) {
+        const int d = dx ? 0 : dy ? 1 : 2;
+        nbor[6 * o + 2 * d + (dx + dy + dz > 0)] = cid;
     }
 }
 
@@ -353,9 +382,12 @@ __global__ void k_tile_counts(BuildView b, const int32_t *__restrict__ pos, int 
 
 // Stencil slots of each tile: a depth-D tile covers 2^D x 2^D x 2^D level-l octs and
 // its stencil (2^D + 2)^3 oct positions, one layer of octs (two cells) around it; the
-// eight corner positions are marked unneeded.
+// eight corner positions are marked unneeded.  The level-(l-1) cell at a position is found
+// from the root's 27 neighbour octs (one level of sons further down for depth 2); the root of
+// the whole tree, whose row has no wrap, searches (as every slot did: 110 us per depth at 0.43 M
+// octs).
 __global__ void k_tile_slots(BuildView b, int depth, int64_t ntile, const int32_t *__restrict__ root,
-                             const int32_t *__restrict__ son, int32_t *slot)
+                             const int32_t *__restrict__ son, const int32_t *__restrict__ nb27, int32_t *slot)
 {
     const int ns = (1 << depth) + 2, nsl = ns * ns * ns;
     const int64_t gi = blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
@@ -369,6 +401,25 @@ __global__ void k_tile_slots(BuildView b, int depth, int64_t ntile, const int32_
     // predicted states of face neighbours only), so they get no ghost father either
     if (int(sx == 0 || sx == ns - 1) + int(sy == 0 || sy == ns - 1) + int(sz == 0 || sz == ns - 1) == 3) {
         slot[gi] = UNNEEDED;
+        return;
+    }
+    if (b.lvl[r] > 1) {
+        // position from the root's corner in level-(l-1) cells, the neighbour oct of the root's
+        // level it lies in, and its place in that oct (2^depth cells of level l-1 per axis)
+        const int w = 1 << depth, rx = sx - 1 + w, ry = sy - 1 + w, rz = sz - 1 + w;
+        const int32_t po = nb27[27 * int64_t(r) + (rx >> depth) + 3 * (ry >> depth) + 9 * (rz >> depth)];
+        int32_t v = OUTSIDE;
+        if (po != OUTSIDE) {
+            v = UNNEEDED;                           // no updated oct of the tile reaches it (2:1 rule)
+            int32_t o = po;                         // the oct of level l-1 (below po's cell, for depth 2)
+            if (depth == 2 && o >= 0) o = son[o * 8 + ((rx >> 1) & 1) + 2 * ((ry >> 1) & 1) + 4 * ((rz >> 1) & 1)];
+            if (o >= 0) {
+                const int32_t F = o * 8 + (rx & 1) + 2 * (ry & 1) + 4 * (rz & 1);
+                const int32_t sn = son[F];
+                v = sn >= 0 ? sn : -1 - F;
+            }
+        }
+        slot[gi] = v;
         return;
     }
     // level-l oct coordinates == level-(l-1) father cell coordinates
@@ -698,16 +749,17 @@ static amr_status build_tree(const amr_geom *geom, const int32_t *h_lxyz, const 
         unsigned long long *hist = (unsigned long long *)(S + W.small + 1024);
         unsigned long long hh[AMR_MAXLEV + 2];
         AMR_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(hh), st));
-        k_level_hist<<<nb, TB, 0, st>>>(lxyz, n, hist);
+        k_level_hist<<<nb < 1216 ? nb : 1216, 256, 0, st>>>(lxyz, n, hist);
         AMR_CUDA_TRY(cudaMemcpyAsync(hh, hist, sizeof(hh), cudaMemcpyDeviceToHost, st));
         AMR_CUDA_TRY(cudaStreamSynchronize(st));
         for (int l = 0; l < AMR_MAXLEV + 2; ++l)
             if (int64_t(hh[l]) != (l <= AMR_MAXLEV ? cnt[l] : 0)) return AMR_EINVAL;
     }
-    k_keys<<<nb, TB, 0, st>>>(lxyz, n, sk0, id0, err);
+    const int kb = 3 * (lmax - 1);                 // at most 57; the level takes five bits above
+    k_keys<<<nb, TB, 0, st>>>(lxyz, n, kb, sk0, id0, err);
     size_t cb = W.cub_bytes;
-    AMR_CUDA_TRY(cub::DeviceRadixSort::SortPairs(cubtmp, cb, sk0, sk1, id0, id1, (int)n, 0, 64, st));
-    k_scatter<<<nb, TB, 0, st>>>(sk1, id1, lxyz, n, out->lvl, out->ix, out->iy, out->iz, out->key, err);
+    AMR_CUDA_TRY(cub::DeviceRadixSort::SortPairs(cubtmp, cb, sk0, sk1, id0, id1, (int)n, 0, kb + 5, st));
+    k_scatter<<<nb, TB, 0, st>>>(sk1, id1, lxyz, n, kb, out->lvl, out->ix, out->iy, out->iz, out->key, err);
 
     BuildView bv;
     bv.n = n; bv.levelmin = lmin; bv.levelmax = lmax;
@@ -721,12 +773,12 @@ static amr_status build_tree(const amr_geom *geom, const int32_t *h_lxyz, const 
     {
         const int64_t o12 = out->lvl_off[3 <= AMR_MAXLEV + 1 ? 3 : AMR_MAXLEV + 1];
         if (o12 > 0)
-            k_tables<<<unsigned((o12 + TB - 1) / TB), TB, 0, st>>>(bv, o12, out->son, out->father, out->nbor,
+            k_tables<<<unsigned((32 * o12 + TB - 1) / TB), TB, 0, st>>>(bv, o12, out->son, out->father, out->nbor,
                                                                     out->nb27, out->refmask, err);
         for (int l = 3; l <= lmax; ++l) {
             const int64_t nl = out->lvl_off[l + 1] - out->lvl_off[l];
             if (nl > 0)
-                k_tables_level<<<unsigned((nl + TB - 1) / TB), TB, 0, st>>>(bv, l, out->son, out->father, out->nbor,
+                k_tables_level<<<unsigned((27 * nl + TB - 1) / TB), TB, 0, st>>>(bv, l, out->son, out->father, out->nbor,
                                                                          out->nb27, out->refmask, err);
         }
     }
@@ -764,7 +816,7 @@ static amr_status build_tree(const amr_geom *geom, const int32_t *h_lxyz, const 
         if (ntile > 0) {
             const int64_t tot = ntile * nslot(d + 1);
             k_tile_slots<<<unsigned((tot + TB - 1) / TB), TB, 0, st>>>(bv, d + 1, ntile, out->tile_root[d], out->son,
-                                                                      out->tile_slot[d]);
+                                                                      out->nb27, out->tile_slot[d]);
         }
     }
     // the reflux pass's work list: per level, in cell order
