@@ -111,7 +111,9 @@ struct TrainSmem {
     float sx[8][16 * 8];
     float sy[8][16 * 2];
     float loss[8];
+    __align__(16) unsigned char packed[PACKED_BYTES];   // the weight block
 };
+static_assert(PACKED_BYTES % 16 == 0, "copied in 16-byte pieces");
 
 // tiles of dW for layer L: (m-tiles of outputs) x (n-tiles of inputs + ones row)
 template <int L> struct Lay;
@@ -205,7 +207,17 @@ __global__ void __launch_bounds__(256, 1) k_train_grad(const void *packed, const
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     TrainSmem &sm = *reinterpret_cast<TrainSmem *>(smraw);
-    const Packed P = view(packed);
+    // the weights once into shared memory: every fragment of the chain below would otherwise
+    // wait for L2 at its first use (a batch of 4096 gives a CTA one chunk)
+    if ((reinterpret_cast<uintptr_t>(packed) & 15) == 0) {
+        for (int j = threadIdx.x; j < int(PACKED_BYTES / 16); j += blockDim.x)
+            reinterpret_cast<uint4 *>(sm.packed)[j] = static_cast<const uint4 *>(packed)[j];
+    } else {
+        for (int j = threadIdx.x; j < int(PACKED_BYTES / 4); j += blockDim.x)
+            reinterpret_cast<uint32_t *>(sm.packed)[j] = static_cast<const uint32_t *>(packed)[j];
+    }
+    __syncthreads();
+    const Packed P = view(sm.packed);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     // constant rows of a^T: the ones row (64 for layers 2-4; 7 for layer 1 is set per chunk)
     for (int j = threadIdx.x; j < 8 * TS; j += blockDim.x) sm.aT[64 + j / TS][j % TS] = __float2bfloat16_rn(j / TS == 0 ? 1.0f : 0.0f);
@@ -334,35 +346,89 @@ __global__ void __launch_bounds__(256, 1) k_train_grad(const void *packed, const
     }
 }
 
-// sum the per-CTA partials in CTA order; entries no tile wrote stay 0 (cleared first)
-__global__ void k_grad_reduce(const float *__restrict__ partial, int nblk, float *grad, const float *__restrict__ lp,
-                              float *loss)
+// the sum of the per-CTA partials of parameter i in CTA order, eight loads in flight
+__device__ __forceinline__ float grad_sum(const float *__restrict__ partial, int nblk, int i)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < NPARAM) {
-        float s = 0.0f;
-        for (int b = 0; b < nblk; ++b) s += partial[int64_t(b) * NPARAM + i];
-        grad[i] = s;
+    float s = 0.0f;
+    int b = 0;
+    for (; b + 8 <= nblk; b += 8) {
+        float p[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) p[k] = partial[int64_t(b + k) * NPARAM + i];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s += p[k];
     }
-    if (i == 0 && loss) {
-        float s = 0.0f;
-        for (int b = 0; b < nblk; ++b) s += lp[b];
-        *loss = s;
-    }
+    for (; b < nblk; ++b) s += partial[int64_t(b) * NPARAM + i];
+    return s;
 }
 
-// Adam (Kingma & Ba 2015) on the FP32 master parameters; t counts from 1
-__global__ void k_adam(float *th, float *m, float *v, const float *__restrict__ grad, float lr, float b1, float b2,
-                       float eps, float c1, float c2)
+__device__ __forceinline__ void loss_sum(const float *__restrict__ lp, int nblk, float *loss)
+{
+    float s = 0.0f;
+    for (int b = 0; b < nblk; ++b) s += lp[b];
+    *loss = s;
+}
+
+__global__ void k_grad_reduce(const float *__restrict__ partial, int nblk, float *grad)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < NPARAM) grad[i] = grad_sum(partial, nblk, i);
+}
+
+// whether entry i of the packed matrices is padding (k_pack writes a zero there)
+__device__ __forceinline__ bool packed_padding(int i)
+{
+    if (i < PW2) return i % S1 >= NIN;
+    if (i < PW4) return (i - PW2) % S >= H;
+    if (i < PW2T) return (i - PW4) / S >= NOUT || (i - PW4) % S >= H;
+    if (i < PW4T) return (i - PW2T) % S >= H;
+    return (i - PW4T) % S4T >= NOUT;
+}
+
+// The end of a training step in one launch: the gradient's sum, Adam (Kingma & Ba 2015; t
+// counts from 1) on the FP32 master parameters, and each new parameter's places in the packed
+// block.  As four launches (clear, sum, Adam, pack) these took as long as the gradient itself.
+__global__ void __launch_bounds__(64) k_train_update(const float *__restrict__ partial, int nblk, float *th, float *m,
+                                                     float *v, __nv_bfloat16 *w, float *bias,
+                                                     const float *__restrict__ lp, float *loss, float lr, float b1,
+                                                     float b2, float eps, float c1, float c2)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i == 0 && loss) loss_sum(lp, nblk, loss);
+    if (i < PEND && packed_padding(i)) w[i] = __float2bfloat16_rn(0.0f);
+    if (i < 8 - NOUT) bias[3 * H + NOUT + i] = 0.0f;
     if (i >= NPARAM) return;
-    const float gr = grad[i];
+    const float gr = grad_sum(partial, nblk, i);
     const float mi = b1 * m[i] + (1.0f - b1) * gr;
     const float vi = b2 * v[i] + (1.0f - b2) * gr * gr;
     m[i] = mi;
     v[i] = vi;
-    th[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float t = th[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    th[i] = t;
+    const __nv_bfloat16 q = __float2bfloat16_rn(t);
+    if (i < OB1) {
+        w[PW1 + (i / NIN) * S1 + i % NIN] = q;
+    } else if (i < OW2) {
+        bias[i - OB1] = t;
+    } else if (i < OB2) {
+        const int j = i - OW2, n = j / H, k = j % H;
+        w[PW2 + n * S + k] = q;
+        w[PW2T + k * S + n] = q;
+    } else if (i < OW3) {
+        bias[H + i - OB2] = t;
+    } else if (i < OB3) {
+        const int j = i - OW3, n = j / H, k = j % H;
+        w[PW3 + n * S + k] = q;
+        w[PW3T + k * S + n] = q;
+    } else if (i < OW4) {
+        bias[2 * H + i - OB3] = t;
+    } else if (i < OB4) {
+        const int j = i - OW4, n = j / H, k = j % H;
+        w[PW4 + n * S + k] = q;
+        w[PW4T + k * S4T + n] = q;
+    } else {
+        bias[3 * H + i - OB4] = t;
+    }
 }
 
 static int grad_blocks(int64_t n)
@@ -417,18 +483,15 @@ extern "C" amr_status mlp_forward(const void *d_packed, const float *d_x, float 
     return AMR_OK;
 }
 
+// the per-CTA partial gradients and losses (every entry of a partial is written by one tile)
 static amr_status grad_launch(const void *d_packed, const float *d_x, const float *d_t, int64_t n, int mode,
-                              float *d_grad, float *d_loss, float *d_scratch, size_t scratch_bytes, cudaStream_t st)
+                              float *d_scratch, size_t scratch_bytes, cudaStream_t st)
 {
     if (scratch_bytes < mlp_scratch_bytes(n)) return AMR_ECAPACITY;
     const int nb = grad_blocks(n);
-    float *partial = d_scratch, *lp = d_scratch + size_t(nb) * mlp::NPARAM;
-    AMR_CUDA_TRY(cudaMemsetAsync(partial, 0, size_t(nb) * mlp::NPARAM * sizeof(float), st));
     const size_t smem = sizeof(TrainSmem);
     AMR_CUDA_TRY(cudaFuncSetAttribute(k_train_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    k_train_grad<<<nb, 256, smem, st>>>(d_packed, d_x, d_t, n, mode, partial, lp);
-    AMR_CUDA_TRY(cudaGetLastError());
-    k_grad_reduce<<<(mlp::NPARAM + 255) / 256, 256, 0, st>>>(partial, nb, d_grad, lp, d_loss);
+    k_train_grad<<<nb, 256, smem, st>>>(d_packed, d_x, d_t, n, mode, d_scratch, d_scratch + size_t(nb) * mlp::NPARAM);
     AMR_CUDA_TRY(cudaGetLastError());
     return AMR_OK;
 }
@@ -437,8 +500,12 @@ extern "C" amr_status mlp_grad(const void *d_packed, const float *d_x, const flo
                                float *d_scratch, size_t scratch_bytes, amr_stream stream)
 {
     if (!d_packed || !d_x || !d_dy || !d_grad || !d_scratch || n <= 0) return AMR_EINVAL;
-    return grad_launch(d_packed, d_x, d_dy, n, 1, d_grad, nullptr, d_scratch, scratch_bytes,
-                       reinterpret_cast<cudaStream_t>(stream));
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    const amr_status r = grad_launch(d_packed, d_x, d_dy, n, 1, d_scratch, scratch_bytes, st);
+    if (r != AMR_OK) return r;
+    k_grad_reduce<<<(mlp::NPARAM + 255) / 256, 256, 0, st>>>(d_scratch, grad_blocks(n), d_grad);
+    AMR_CUDA_TRY(cudaGetLastError());
+    return AMR_OK;
 }
 
 extern "C" amr_status mlp_train_step(float *d_theta, float *d_adam_m, float *d_adam_v, void *d_packed,
@@ -448,12 +515,18 @@ extern "C" amr_status mlp_train_step(float *d_theta, float *d_adam_m, float *d_a
     if (!d_theta || !d_adam_m || !d_adam_v || !d_packed || !d_x || !d_y || !d_scratch || n <= 0 || t < 1)
         return AMR_EINVAL;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    float *grad = d_scratch + size_t(grad_blocks(n)) * (mlp::NPARAM + 1);
-    amr_status r = grad_launch(d_packed, d_x, d_y, n, 0, grad, d_loss, d_scratch, scratch_bytes, st);
+    if (uintptr_t(d_packed) & 15) return AMR_EINVAL;
+    const amr_status r = grad_launch(d_packed, d_x, d_y, n, 0, d_scratch, scratch_bytes, st);
     if (r != AMR_OK) return r;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, float(t)), c2 = 1.0f - powf(b2, float(t));
-    k_adam<<<(mlp::NPARAM + 255) / 256, 256, 0, st>>>(d_theta, d_adam_m, d_adam_v, grad, lr, b1, b2, 1e-8f, c1, c2);
+    const int nb = grad_blocks(n);
+    const Packed P = view(d_packed);
+    static_assert(mlp::PEND >= mlp::NPARAM, "a thread per packed entry covers the parameters");
+    k_train_update<<<(mlp::PEND + 63) / 64, 64, 0, st>>>(d_scratch, nb, d_theta, d_adam_m, d_adam_v,
+                                                         const_cast<__nv_bfloat16 *>(P.w), const_cast<float *>(P.b),
+                                                         d_scratch + size_t(nb) * mlp::NPARAM, d_loss, lr, b1, b2,
+                                                         1e-8f, c1, c2);
     AMR_CUDA_TRY(cudaGetLastError());
-    return mlp_pack(d_theta, d_packed, stream);
+    return AMR_OK;
 }
