@@ -15,7 +15,10 @@ amr_status harvest_dispatch(const amr_tree *t, const hydro_params *p, const doub
 amr_status godunov_dispatch_fp64(const amr_tree *t, int level, const hydro_params *p, const double *u_old,
                                  double *u_new, double *reg, const double *dt, double *dt_next, cudaStream_t st);
 
-// warp minimum of positive doubles (compared as their bit patterns), then one atomic per warp
+// warp minimum of positive doubles (compared as their bit patterns), then at most one atomic
+// per warp: none when the target already holds a smaller value (it only falls, so a stale read
+// costs no more than an atomic that changes nothing).  An atomic per warp serialised on the one
+// address: 597 us for the 18.9 M cells of a 256^3 tree.
 __device__ __forceinline__ void min_to(double *target, double v)
 {
     unsigned long long b = v < DBL_MAX ? (unsigned long long)__double_as_longlong(v) : ~0ull;
@@ -23,7 +26,10 @@ __device__ __forceinline__ void min_to(double *target, double v)
         const unsigned long long o = __shfl_xor_sync(0xffffffffu, b, off);
         b = o < b ? o : b;
     }
-    if ((threadIdx.x & 31) == 0 && b != ~0ull) atomicMin(reinterpret_cast<unsigned long long *>(target), b);
+    if ((threadIdx.x & 31) == 0 && b != ~0ull) {
+        unsigned long long *t = reinterpret_cast<unsigned long long *>(target);
+        if (b < *reinterpret_cast<volatile unsigned long long *>(t)) atomicMin(t, b);
+    }
 }
 
 template <typename R>
@@ -53,16 +59,18 @@ __global__ void k_dt_levels(const double *__restrict__ dt_base, int levelmin, do
     if (l < AMR_MAXLEV + 2) dtl[l] = l > levelmin ? scale_pow2(*dt_base, levelmin - l) : *dt_base;
 }
 
-// sub-cycling: leaves of one level take the mean of two states (time interpolation)
-__global__ void k_lerp_leaves(TreeView tv, int level, double *U, const double *__restrict__ N)
+// sub-cycling: n consecutive cells of each variable (n even), one launch instead of a copy per
+// variable
+__global__ void __launch_bounds__(256) k_copy_level(const double *__restrict__ src, double *__restrict__ dst, int64_t n,
+                                                    int64_t ncell)
 {
-    const int64_t cell = tv.lvl_off[level] * 8 + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
-    if (cell >= tv.lvl_off[level + 1] * 8 || tv.son[cell] >= 0) return;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int64_t i = v * tv.ncell + cell;
-        U[i] = 0.5 * (U[i] + N[i]);
-    }
+    const int64_t i = 2 * (blockIdx.x * int64_t(blockDim.x) + threadIdx.x);
+    if (i >= n) return;
+    const double *s = src + blockIdx.y * ncell + i;
+    double *d = dst + blockIdx.y * ncell + i;
+    const double a = s[0], b = s[1];
+    d[0] = a;
+    d[1] = b;
 }
 
 // batch mode: per-box CFL step (box cell ranges are multiples of 64, so a warp never
@@ -84,6 +92,43 @@ __global__ void k_courant_batch(TreeView tv, const double *__restrict__ u, doubl
     }
     b = __shfl_sync(0xffffffffu, b, 0);
     min_to(dt + b, cand);
+}
+
+// The correction of leaf `cell` of a coarse level by the fine fluxes of its refined face
+// neighbours (-/+ dt/dx * 1/4 * sum of the four fine fluxes), added to the state A and, if
+// given, to a second state B; whether there was one.
+__device__ __forceinline__ bool reflux_leaf(const TreeView &tv, int level, int64_t cell,
+                                            const double *__restrict__ reg, const double *dtp, double A[NV], double *B)
+{
+    const int64_t o = cell >> 3;
+    const int c = int(cell & 7);
+    const double lam = scale_pow2(*dtp, level);   // dt / dx, exact
+    bool hit = false;
+    for (int f = 0; f < 6; ++f) {
+        const int d = f >> 1, side = f & 1;
+        int64_t nb;
+        if (((c >> d) & 1) != side) {
+            nb = o * 8 + (c ^ (1 << d));
+        } else {
+            const int32_t N = tv.nbor[6 * o + f];
+            if (N < 0) continue;                      // outflow face of the box
+            const int32_t so = tv.son[N];
+            if (so < 0) continue;                     // coarser neighbour
+            nb = int64_t(so) * 8 + (c ^ (1 << d));
+        }
+        const int32_t fo = tv.son[nb];
+        if (fo < 0) continue;
+        const int opp = 2 * d + (1 - side);
+        const double *rrow = reg + ((int64_t(fo) - tv.reg_base) * 6 + opp) * NV;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const double corr = 0.25 * rrow[v];
+            A[v] = side ? A[v] - lam * corr : A[v] + lam * corr;
+            if (B) B[v] = side ? B[v] - lam * corr : B[v] + lam * corr;
+        }
+        hit = true;
+    }
+    return hit;
 }
 
 // Coarse level l: leaf cells next to a refined cell take the fine fluxes from the
@@ -110,34 +155,10 @@ __device__ __forceinline__ double reflux_cell(const TreeView &tv, int level, int
             }
         }
     } else if (reg && level >= tv.levelmin) {
-        const double lam = scale_pow2(*dtp, level);   // dt / dx, exact
         double U[NV];
 #pragma unroll
         for (int v = 0; v < NV; ++v) U[v] = u[v * tv.ncell + cell];
-        bool hit = false;
-        for (int f = 0; f < 6; ++f) {
-            const int d = f >> 1, side = f & 1;
-            int64_t nb;
-            if (((c >> d) & 1) != side) {
-                nb = o * 8 + (c ^ (1 << d));
-            } else {
-                const int32_t N = tv.nbor[6 * o + f];
-                if (N < 0) continue;                      // outflow face of the box
-                const int32_t so = tv.son[N];
-                if (so < 0) continue;                     // coarser neighbour
-                nb = int64_t(so) * 8 + (c ^ (1 << d));
-            }
-            const int32_t fo = tv.son[nb];
-            if (fo < 0) continue;
-            const int opp = 2 * d + (1 - side);
-            const double *rrow = reg + ((int64_t(fo) - tv.reg_base) * 6 + opp) * NV;
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                const double corr = 0.25 * rrow[v];
-                U[v] = side ? U[v] - lam * corr : U[v] + lam * corr;
-            }
-            hit = true;
-        }
+        const bool hit = reflux_leaf(tv, level, cell, reg, dtp, U, static_cast<double *>(nullptr));
         if (hit) {
 #pragma unroll
             for (int v = 0; v < NV; ++v) u[v * tv.ncell + cell] = U[v];
@@ -159,6 +180,48 @@ __global__ void k_reflux(TreeView tv, int level, const double *__restrict__ reg,
     if (cell < tv.lvl_off[level + 1] * 8)
         cand = reflux_cell<R>(tv, level, cell, reg, u, dtp, dt_next != nullptr, gamma, rf, pf, cfl, restrict_all);
     if (dt_next) min_to(dt_next, cand);
+}
+
+// Sub-cycling, between the two fine steps of level + 1: the ghosts' state U of this level
+// becomes the mean of its start and end states plus the first fine step's correction in the
+// leaves and the mean of the children in the refined cells; the end state N takes the
+// correction in the leaves and, where the update kernel has not restricted, the mean of its
+// children.  One pass over the level in place of an interpolation, a full and a listed reflux
+// pass (18 + 23 + 15 us on a level of 2 M cells).
+__global__ void __launch_bounds__(256) k_sc_middle(TreeView tv, int level, const double *__restrict__ reg, double *U,
+                                                   double *N, const double *dtp)
+{
+    const int64_t cell = tv.lvl_off[level] * 8 + blockIdx.x * int64_t(blockDim.x) + threadIdx.x;
+    if (cell >= tv.lvl_off[level + 1] * 8) return;
+    const int32_t s = tv.son[cell];
+    if (s >= 0) {
+        const bool both = !tv.fused[s];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            double su = 0.0, sn = 0.0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) su += U[v * tv.ncell + int64_t(s) * 8 + q];
+            U[v * tv.ncell + cell] = 0.125 * su;
+            if (both) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) sn += N[v * tv.ncell + int64_t(s) * 8 + q];
+                N[v * tv.ncell + cell] = 0.125 * sn;
+            }
+        }
+        return;
+    }
+    double u[NV], n[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        n[v] = N[v * tv.ncell + cell];
+        u[v] = 0.5 * (U[v * tv.ncell + cell] + n[v]);
+    }
+    if (reflux_leaf(tv, level, cell, reg, dtp, u, n)) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) N[v * tv.ncell + cell] = n[v];
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) U[v * tv.ncell + cell] = u[v];
 }
 
 // The same pass over the cells of the tree's work list of one level only (the others have
@@ -455,20 +518,18 @@ static amr_status sc_advance(const amr_tree *t, const hydro_params *p, int c, do
         // fine step's correction; refined cells restricted from the fine level
         const int64_t nc = (t->lvl_off[c + 1] - t->lvl_off[c]) * 8;
         if (nc > 0) {
-            k_lerp_leaves<<<unsigned((nc + 255) / 256), 256, 0, st>>>(make_view(t), c, U, N);
+            k_sc_middle<<<unsigned((nc + 255) / 256), 256, 0, st>>>(make_view(t), c, reg, U, N, dtl + c + 1);
             AMR_CUDA_TRY(cudaGetLastError());
         }
-        if ((r = reflux_launch(t, c, p, reg, U, dtl + c + 1, nullptr, st, 1)) != AMR_OK) return r;
-        if ((r = reflux_launch(t, c, p, reg, N, dtl + c + 1, nullptr, st, 0)) != AMR_OK) return r;
         if ((r = sc_advance(t, p, c + 1, U, N, reg, dtl, st)) != AMR_OK) return r;
         if ((r = reflux_launch(t, c, p, reg, N, dtl + c + 1, nullptr, st, 0)) != AMR_OK) return r;
     }
     // the level's new state becomes current (its cells are contiguous in each variable)
     const int64_t c0 = t->lvl_off[c] * 8, n = (t->lvl_off[c + 1] - t->lvl_off[c]) * 8, ncell = 8 * t->noct;
-    if (n > 0)
-        for (int v = 0; v < NV; ++v)
-            AMR_CUDA_TRY(cudaMemcpyAsync(U + v * ncell + c0, N + v * ncell + c0, size_t(n) * sizeof(double),
-                                         cudaMemcpyDeviceToDevice, st));
+    if (n > 0) {
+        k_copy_level<<<dim3(unsigned((n / 2 + 255) / 256), NV), 256, 0, st>>>(N + c0, U + c0, n, ncell);
+        AMR_CUDA_TRY(cudaGetLastError());
+    }
     return AMR_OK;
 }
 
@@ -503,9 +564,7 @@ extern "C" amr_status hydro_step_subcycled(const amr_tree *t, const hydro_params
     k_dt_levels<<<1, 32, 0, st>>>(d_dt, t->levelmin, d_dt_levels);
     AMR_CUDA_TRY(cudaGetLastError());
     if ((r = sc_advance(t, p, t->levelmin, d_u, d_scratch, d_flux_reg, d_dt_levels, st)) != AMR_OK) return r;
-    for (int l = t->levelmin - 1; l >= 1; --l)
-        if ((r = reflux_launch(t, l, p, nullptr, d_u, d_dt_levels, nullptr, st, 1)) != AMR_OK) return r;
-    return AMR_OK;
+    return restrict_complete_launch(t, t->levelmin, d_u, st);
 }
 
 extern "C" amr_status hydro_restrict_complete(const amr_tree *t, double *d_u, amr_stream stream)
