@@ -209,57 +209,73 @@ struct Smem {
 };
 static_assert(Geo<2>::NSLOT <= 256, "slot indices fit a byte");
 
-// left and right states of face r0 of direction DIR (face-normal frame), floored
-template <typename R, int D, int RS, int DIR>
-__device__ __forceinline__ void face_states(const Smem<R, D, RS> &sm, int r0, const Prm<R> &pr, R WL[NV], R WR[NV])
+// A face of the tile: direction d, face r0 of it, its place among the fluxes.  The direction is
+// a value, not a template argument: one copy of the Riemann solve instead of three (the launch
+// stalled on instruction fetch), and a warp whose faces straddle two directions solves once.
+struct TileFace {
+    int d, r0;
+    int N0, T1, T2;      // normal and transverse velocity components
+};
+template <int D> __device__ __forceinline__ TileFace tile_face(int f)
 {
     using G = Geo<D>;
-    const int fa = r0 % (G::CI + 1), t1 = (r0 / (G::CI + 1)) % G::CI, t2 = r0 / ((G::CI + 1) * G::CI);
-    const int Lx = DIR == 0 ? fa : 1 + t1;
-    const int Ly = DIR == 0 ? 1 + t1 : DIR == 1 ? fa : 1 + t2;
-    const int Lz = DIR == 2 ? fa : 1 + t2;
-    const int pl = Lx + G::P * (Ly + G::P * Lz);
-    const int pR = pl + (DIR == 0 ? 1 : DIR == 1 ? G::P : G::P * G::P);
-    constexpr int S = NV + NV * DIR;
-    R tL[NV], dL[NV], tR[NV], dR[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        tL[v] = sm.Q[v][pl]; dL[v] = sm.Q[S + v][pl];
-        tR[v] = sm.Q[v][pR]; dR[v] = sm.Q[S + v][pR];
-    }
-    face_state<DIR>(tL, dL, R(0.5), pr, WL);
-    face_state<DIR>(tR, dR, R(-0.5), pr, WR);
+    TileFace t;
+    t.d = f / G::NF;
+    t.r0 = f - t.d * G::NF;
+    t.N0 = t.d + 1;
+    t.T1 = t.d == 0 ? 2 : 1;
+    t.T2 = t.d == 2 ? 2 : 3;
+    return t;
 }
 
-template <typename R, int D, int RS, int DIR>
-__device__ __forceinline__ void face_flux(Smem<R, D, RS> &sm, R (*sF)[NV][Geo<D>::NF], int r0, const Prm<R> &pr,
+// left and right states of a face (face-normal frame), floored
+template <typename R, int D, int RS>
+__device__ __forceinline__ void face_states(const Smem<R, D, RS> &sm, const TileFace &t, const Prm<R> &pr, R WL[NV],
+                                            R WR[NV])
+{
+    using G = Geo<D>;
+    const int fa = t.r0 % (G::CI + 1), t1 = (t.r0 / (G::CI + 1)) % G::CI, t2 = t.r0 / ((G::CI + 1) * G::CI);
+    // predicted-cell coordinates (stencil - 1) of the left cell
+    const int Lx = t.d == 0 ? fa : 1 + t1;
+    const int Ly = t.d == 0 ? 1 + t1 : t.d == 1 ? fa : 1 + t2;
+    const int Lz = t.d == 2 ? fa : 1 + t2;
+    const int pl = Lx + G::P * (Ly + G::P * Lz);
+    const int pR = pl + (t.d == 0 ? 1 : t.d == 1 ? G::P : G::P * G::P);
+    const R *q = &sm.Q[0][0], *dq = &sm.Q[NV + NV * t.d][0];
+    const int row[NV] = {0, t.N0 * G::NP, t.T1 * G::NP, t.T2 * G::NP, 4 * G::NP};
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        WL[v] = fmar(R(0.5), dq[row[v] + pl], q[row[v] + pl]);
+        WR[v] = fmar(R(-0.5), dq[row[v] + pR], q[row[v] + pR]);
+    }
+    WL[0] = rmax(WL[0], pr.rho_floor);
+    WR[0] = rmax(WR[0], pr.rho_floor);
+    WL[4] = rmax(WL[4], pr.p_floor);
+    WR[4] = rmax(WR[4], pr.p_floor);
+}
+
+template <int D, typename R>
+__device__ __forceinline__ void face_store(R (*sF)[NV][Geo<D>::NF], const TileFace &t, const R Fn[NV])
+{
+    R *o = &sF[t.d][0][t.r0];
+    o[0] = Fn[0];
+    o[t.N0 * Geo<D>::NF] = Fn[1];
+    o[t.T1 * Geo<D>::NF] = Fn[2];
+    o[t.T2 * Geo<D>::NF] = Fn[3];
+    o[4 * Geo<D>::NF] = Fn[4];
+}
+
+template <typename R, int D, int RS>
+__device__ __forceinline__ void face_flux(Smem<R, D, RS> &sm, R (*sF)[NV][Geo<D>::NF], int f, const Prm<R> &pr,
                                           int32_t *status, const GArgs &a, int64_t tile, unsigned &n_it,
                                           unsigned &n_solve)
 {
-    using G = Geo<D>;
-    const int fa = r0 % (G::CI + 1), t1 = (r0 / (G::CI + 1)) % G::CI, t2 = r0 / ((G::CI + 1) * G::CI);
-    // predicted-cell coordinates (stencil - 1) of the left cell
-    const int Lx = DIR == 0 ? fa : 1 + t1;
-    const int Ly = DIR == 0 ? 1 + t1 : DIR == 1 ? fa : 1 + t2;
-    const int Lz = DIR == 2 ? fa : 1 + t2;
-    const int pl = Lx + G::P * (Ly + G::P * Lz);
-    const int pR = pl + (DIR == 0 ? 1 : DIR == 1 ? G::P : G::P * G::P);
-    constexpr int N0 = DIR + 1, T1 = DIR == 0 ? 2 : 1, T2 = DIR == 2 ? 2 : 3;   // normal, transverse
-    constexpr int S = NV + NV * DIR;                                             // slopes along DIR
+    const TileFace t = tile_face<D>(f);
     R WL[NV], WR[NV];
-    {
-        R tL[NV], dL[NV], tR[NV], dR[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            tL[v] = sm.Q[v][pl]; dL[v] = sm.Q[S + v][pl];
-            tR[v] = sm.Q[v][pR]; dR[v] = sm.Q[S + v][pR];
-        }
-        face_state<DIR>(tL, dL, R(0.5), pr, WL);
-        face_state<DIR>(tR, dR, R(-0.5), pr, WR);
-    }
+    face_states<R, D, RS>(sm, t, pr, WL, WR);
     if (a.harvest) {
         // deterministic sample of the faces (hash of tile, direction and face)
-        uint64_t h = (uint64_t(tile) * 3 + DIR) * 0x9E3779B97F4A7C15ull + uint64_t(r0) * 0xBF58476D1CE4E5B9ull;
+        uint64_t h = (uint64_t(tile) * 3 + t.d) * 0x9E3779B97F4A7C15ull + uint64_t(t.r0) * 0xBF58476D1CE4E5B9ull;
         h ^= h >> 31;
         if (h % uint64_t(a.harvest_stride) == 0) {
             const unsigned long long k = atomicAdd(a.harvest_count, 1ull);
@@ -290,11 +306,7 @@ __device__ __forceinline__ void face_flux(Smem<R, D, RS> &sm, R (*sF)[NV][Geo<D>
     } else {
         hllc(WL, WR, pr, Fn);
     }
-    sF[DIR][0][r0] = Fn[0];
-    sF[DIR][N0][r0] = Fn[1];
-    sF[DIR][T1][r0] = Fn[2];
-    sF[DIR][T2][r0] = Fn[3];
-    sF[DIR][4][r0] = Fn[4];
+    face_store<D>(sF, t, Fn);
 }
 
 
@@ -316,11 +328,9 @@ __device__ __forceinline__ void mlp_faces(Smem<R, D, RS> &sm, R (*sF)[NV][Geo<D>
     for (int base = warp * 32; base < 3 * G::NF; base += nw * 32) {
         const int f = base + lane;
         const bool valid = f < 3 * G::NF;
-        const int d = valid ? f / G::NF : 0, r0 = valid ? f - d * G::NF : 0;
+        const TileFace t = tile_face<D>(valid ? f : 0);
         R WL[NV], WR[NV];
-        if (d == 0) face_states<R, D, RS, 0>(sm, r0, pr, WL, WR);
-        else if (d == 1) face_states<R, D, RS, 1>(sm, r0, pr, WL, WR);
-        else face_states<R, D, RS, 2>(sm, r0, pr, WL, WR);
+        face_states<R, D, RS>(sm, t, pr, WL, WR);
         R x[7], pref, ubar, cref;
         mlp::features(WL[0], WL[1], WL[4], WR[0], WR[1], WR[4], pr.gamma, x, pref, ubar, cref);
 #pragma unroll
@@ -380,14 +390,7 @@ __device__ __forceinline__ void mlp_faces(Smem<R, D, RS> &sm, R (*sF)[NV][Geo<D>
         const unsigned acc = __ballot_sync(0xffffffffu, ok && valid), fb = __ballot_sync(0xffffffffu, !ok && valid);
         n_acc += __popc(acc);
         n_fb += __popc(fb);
-        if (valid) {
-            const int N0 = d + 1, T1 = d == 0 ? 2 : 1, T2 = d == 2 ? 2 : 3;
-            sF[d][0][r0] = Fn[0];
-            sF[d][N0][r0] = Fn[1];
-            sF[d][T1][r0] = Fn[2];
-            sF[d][T2][r0] = Fn[3];
-            sF[d][4][r0] = Fn[4];
-        }
+        if (valid) face_store<D>(sF, t, Fn);
     }
 }
 
@@ -409,6 +412,13 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
 
     unsigned n_acc = 0, n_fb = 0;   // surrogate: accepted faces, fallbacks (counted by lane 0)
     unsigned n_it = 0, n_solve = 0; // Newton iterations and Newton solves of this thread
+    unsigned long long my_dt = ~0ull;   // bit pattern of the smallest positive CFL candidate
+    auto flush_dt = [&](double *target, unsigned long long m) {
+        if (!target) return;
+        for (int off = 16; off > 0; off >>= 1) m = umin64(m, __shfl_xor_sync(0xffffffffu, m, off));
+        unsigned long long *p = reinterpret_cast<unsigned long long *>(target);
+        if ((tid & 31) == 0 && m < *reinterpret_cast<volatile unsigned long long *>(p)) atomicMin(p, m);
+    };
     // The launch has as many CTAs as fit on the GPU at once, each looping over tiles: the
     // next tile's slot entries and refinement masks are loaded into registers while the
     // current tile runs (one slot per thread: NSLOT <= threads).
@@ -524,17 +534,18 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
             const int si = i + G::C * (j + G::C * k);
             const int32_t e = sm.slot[s];
             if (e == OUTSIDE) continue;
-            R Uw[NV];
+            R Uw[NV] = {R(1), R(0), R(0), R(0), R(1)};
             if (e >= 0) {
 #pragma unroll
                 for (int v = 0; v < NV; ++v) Uw[v] = to_work<R>(a.u_old[v * tv.ncell + int64_t(e) * 8 + c]);
             } else if (e == UNNEEDED_SLOT) {
-                Uw[0] = R(1); Uw[1] = R(0); Uw[2] = R(0); Uw[3] = R(0); Uw[4] = R(1);
+                // a placeholder that no face reads
             } else if (a.ghost) {
                 const R *gh = static_cast<const R *>(a.ghost) + (int64_t(-1) - e) * 8 + c;
 #pragma unroll
                 for (int v = 0; v < NV; ++v) Uw[v] = gh[v * a.ghost_stride];
-            } else {
+            } else if constexpr (sizeof(R) == 8) {
+                // the face-state harvest, which has no ghost buffer
                 interp_child<R>(tv, a.u_old, tv.ghost_cell[int64_t(-1) - e], c, Uw);
             }
             R Wc[NV];
@@ -591,16 +602,49 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
 
         if (have_nx && tid < G::NSLOT) rf_nx = e_nx >= 0 ? tv.refmask[e_nx] : 0;
 
+        // what the update and the restriction read from global memory, under way during the
+        // Riemann solves: the old states of the updated cells (into the stencil buffer behind
+        // the fluxes, where there is room) and the restriction's look-ups
+        constexpr size_t FLUX_BYTES = 3 * NV * G::NF * sizeof(R);
+        constexpr bool STAGE = FLUX_BYTES + sizeof(double) * NV * G::NI <= sizeof(sm.W) && G::NI <= threads_for<D>();
+        double(*sO)[G::NI] = reinterpret_cast<double(*)[G::NI]>(reinterpret_cast<char *>(&sm.W[0][0]) +
+                                                                (STAGE ? FLUX_BYTES : 0));
+        constexpr int NRES = G::OI * G::OI * G::OI * NV;
+        static_assert(NRES <= threads_for<D>(), "one restriction item per thread");
+        int32_t r_oct = -1, r_father = 0;
+        uint8_t r_fused = 0;
+        if (!a.harvest) {
+            if (STAGE && tid < G::NI) {
+                const int c = tid & 7, o = tid >> 3;
+                const int sl = (1 + o % G::OI) + G::NS * ((1 + (o / G::OI) % G::OI) + G::NS * (1 + o / (G::OI * G::OI)));
+                const int32_t e = sm.slot[sl];
+                if (e >= 0 && !((sm.ref[sl] >> c) & 1)) {
+                    const double *src = a.u_old + int64_t(e) * 8 + c;
+#pragma unroll
+                    for (int v = 0; v < NV; ++v)
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                                         unsigned(__cvta_generic_to_shared(&sO[v][tid]))),
+                                     "l"(src + v * tv.ncell)
+                                     : "memory");
+                }
+            }
+            // (a box batch restricts nothing and has no father table)
+            if (tid < NRES && !a.tile_inst) {
+                const int o = tid / NV;
+                r_oct = sm.slot[(1 + o % G::OI) + G::NS * ((1 + (o / G::OI) % G::OI) + G::NS * (1 + o / (G::OI * G::OI)))];
+                if (r_oct >= 0) {
+                    r_fused = tv.fused[r_oct];
+                    r_father = tv.father[r_oct];
+                }
+            }
+        }
+
         // ---- phase 3: Riemann problem at every face touching an updated cell
         if constexpr (RS == AMR_RIEMANN_MLP) {
             mlp_faces<R, D, RS>(sm, sF, pr, a, n_acc, n_fb, n_it, n_solve);
         } else {
-            for (int f = tid; f < 3 * G::NF; f += blockDim.x) {
-                const int d = f / G::NF, r0 = f - d * G::NF;
-                if (d == 0) face_flux<R, D, RS, 0>(sm, sF, r0, pr, a.status, a, t, n_it, n_solve);
-                else if (d == 1) face_flux<R, D, RS, 1>(sm, sF, r0, pr, a.status, a, t, n_it, n_solve);
-                else face_flux<R, D, RS, 2>(sm, sF, r0, pr, a.status, a, t, n_it, n_solve);
-            }
+            for (int f = tid; f < 3 * G::NF; f += blockDim.x)
+                face_flux<R, D, RS>(sm, sF, f, pr, a.status, a, t, n_it, n_solve);
         }
         __syncthreads();
         if (a.harvest) continue;   // harvesting only: no update (the loop ends with no barrier due)
@@ -640,7 +684,7 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
         // new states of octs whose father is restricted here, in the (now free) predictor buffer
         double(*sU)[G::NI] = reinterpret_cast<double(*)[G::NI]>(&sm.Q[0][0]);
         static_assert(sizeof(double) * NV * G::NI <= sizeof(R) * 4 * NV * G::NP, "restriction buffer");
-        unsigned long long my_dt = ~0ull;   // bit pattern of the smallest positive candidate
+        if (STAGE) asm volatile("cp.async.wait_all;" ::: "memory");
         for (int q = tid; q < G::NI; q += blockDim.x) {
             const int c = q & 7, o = q >> 3;
             const int ox = 1 + o % G::OI, oy = 1 + (o / G::OI) % G::OI, oz = 1 + o / (G::OI * G::OI);
@@ -679,45 +723,45 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
                 // FP64 accumulation: U_new = U_old + dt/dx * (sum of face fluxes); in the FP32 path
                 // the increment is formed in FP32 (dt/dx is exact there: dt is an FP32 value and
                 // dx a power of two) and added in FP64
-                if (sizeof(R) == 8) Un[v] = a.u_old[v * tv.ncell + cell] + lam * to_state(dU[v]);
-                else Un[v] = a.u_old[v * tv.ncell + cell] + to_state(lamR * dU[v]);
+                const double Uo = STAGE ? sO[v][q] : a.u_old[v * tv.ncell + cell];
+                if constexpr (sizeof(R) == 8) Un[v] = Uo + lam * to_state(dU[v]);
+                else Un[v] = add_f32(Uo, lamR * dU[v]);
                 a.u_new[v * tv.ncell + cell] = Un[v];
+                sU[v][q] = Un[v];                                // kept for the restriction pass
             }
             if (!state_finite<R>(Un)) set_error(a.status, AMR_ENONPHYSICAL);
-            if (tv.fused[e]) {
-#pragma unroll
-                for (int v = 0; v < NV; ++v) sU[v][q] = Un[v];   // kept for the restriction pass
-            }
             if (dtn && !nbref) {
                 // CFL candidate (newdt_fine) from the final new state of this leaf cell
                 const double cand = cfl_candidate<R>(Un, pr, cflR, to_work<R>(dx));
                 my_dt = umin64(my_dt, dbits(cand));
             }
         }
-        if (dtn) {
-            for (int off = 16; off > 0; off >>= 1) my_dt = umin64(my_dt, __shfl_xor_sync(0xffffffffu, my_dt, off));
-            if ((tid & 31) == 0 && my_dt != ~0ull) atomicMin(reinterpret_cast<unsigned long long *>(dtn), my_dt);
+        if (a.tile_inst) {
+            flush_dt(dtn, my_dt);            // boxes have their own time steps
+            my_dt = ~0ull;
         }
 
         // ---- restriction of father cells whose eight children are final here: one thread per
         // (oct, variable), children summed in cell order, so every FP64 lane does useful work
         __syncthreads();
-        for (int w = tid; w < G::OI * G::OI * G::OI * NV; w += blockDim.x) {
-            const int o = w / NV, v = w % NV;
-            const int ox = 1 + o % G::OI, oy = 1 + (o / G::OI) % G::OI, oz = 1 + o / (G::OI * G::OI);
-            const int32_t e = sm.slot[ox + G::NS * (oy + G::NS * oz)];
-            if (e < 0 || !tv.fused[e]) continue;
+        if (tid < NRES && r_oct >= 0 && r_fused) {
+            const int o = tid / NV, v = tid % NV;
             double acc = 0.0;
 #pragma unroll
             for (int c = 0; c < 8; ++c) acc += sU[v][o * 8 + c];
-            a.u_new[v * tv.ncell + tv.father[e]] = 0.125 * acc;
+            a.u_new[v * tv.ncell + r_father] = 0.125 * acc;
         }
 
-        // ---- flux register rows (with depth-1 tiles written above, during the update)
-        if (a.reg && !EARLY_REG)
-            for (int w = tid; w < NREG; w += blockDim.x) reg_task(w);
-        __syncthreads();
+        // ---- flux register rows (with depth-1 tiles written above, during the update).  After
+        // the barrier before the restriction nothing of those reads the slots or the stencil
+        // buffer, and the predictor buffer is next written two barriers on: no barrier here
+        if (!EARLY_REG) {
+            if (a.reg)
+                for (int w = tid; w < NREG; w += blockDim.x) reg_task(w);
+            __syncthreads();
+        }
     }
+    if (!a.tile_inst) flush_dt(a.dt_next, my_dt);
     if (RS == AMR_RIEMANN_MLP && a.counters && (tid & 31) == 0 && (n_acc | n_fb)) {
         atomicAdd(a.counters + 0, (unsigned long long)n_acc);
         atomicAdd(a.counters + 1, (unsigned long long)n_fb);
