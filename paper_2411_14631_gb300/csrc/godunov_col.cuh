@@ -505,14 +505,11 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
     }
 }
 
-// CTAs of a kernel that are resident on the GPU at once
-template <typename K> inline int64_t resident_ctas(K kern, int threads, size_t smem)
+// grid of a z-column kernel: equal shares, one per resident CTA, or segments of a.zc planes
+inline unsigned column_grid(int64_t resident, ColArgs &a)
 {
-    int dev = 0, nsm = 152, per_sm = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    return int64_t(per_sm) * nsm;
+    a.share = a.zc > 0 ? a.zc : even_share(a.planes, resident);
+    return unsigned((a.planes + a.share - 1) / a.share);
 }
 
 template <typename R, int RS>
@@ -545,11 +542,7 @@ amr_status launch_col(const amr_tree *t, const hydro_params *p, const double *u_
     const bool finer = a.finer != 0;
     const size_t bytes = finer ? sizeof(ColSmem<R, FX, FY, true>) : sizeof(ColSmem<R, FX, FY, false>);
     auto kern = finer ? k_godunov_col<R, RS, FX, FY, true> : k_godunov_col<R, RS, FX, FY, false>;
-    AMR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
-    a.share = a.zc > 0 ? a.zc : even_share(a.planes, resident_ctas(kern, 256, bytes));
-    kern<<<unsigned((a.planes + a.share - 1) / a.share), 256, bytes, st>>>(a);
-    AMR_CUDA_TRY(cudaGetLastError());
-    return AMR_OK;
+    return launch_kernel(kern, 256, bytes, false, st, a, column_grid);
 }
 
 }  // namespace amr

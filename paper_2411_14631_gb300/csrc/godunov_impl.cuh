@@ -776,28 +776,17 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
 }
 
 template <typename R, int D, int RS>
-static amr_status launch(const GArgs &a, int64_t ntile, cudaStream_t st)
+static amr_status launch(GArgs &a, int64_t ntile, cudaStream_t st)
 {
     if (ntile <= 0) return AMR_OK;
     // 227 KB per CTA at most; the FP32 depth-1 update keeps eight CTAs in an SM's 228 KB
     // (each with its 1 KB reserved by the system)
     static_assert(sizeof(Smem<R, D, RS>) <= 227 * 1024, "tile shared memory");
     static_assert((sizeof(Smem<R, D, RS>) + 1024) * min_ctas_for<R, D, RS>() <= 228 * 1024, "depth-1 CTAs per SM");
-    const size_t bytes = sizeof(Smem<R, D, RS>);
-    auto kern = k_godunov<R, D, RS>;
-    AMR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
     // as many CTAs as are resident at once (each loops over tiles and prefetches the next
     // tile's slot table)
-    int dev = 0, nsm = 152, per_sm = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads_for<D>(), bytes) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
-    const int64_t resident = int64_t(per_sm) * nsm;
-    const int64_t grid = ntile < resident ? ntile : resident;
-    kern<<<unsigned(grid), threads_for<D>(), bytes, st>>>(a);
-    AMR_CUDA_TRY(cudaGetLastError());
-    return AMR_OK;
+    return launch_kernel(k_godunov<R, D, RS>, threads_for<D>(), sizeof(Smem<R, D, RS>), false, st, a,
+                         [&](int64_t resident, const GArgs &) { return unsigned(ntile < resident ? ntile : resident); });
 }
 
 // The z-column kernel for the deepest complete level (or the box batch): the pencil

@@ -102,7 +102,7 @@ __device__ __forceinline__ void pen_barrier() { asm volatile("bar.sync 1, %0;" :
 // the same for every thread as far as the compiler can see, and stays out of the threads'
 // registers)
 template <int RS, bool FINER, bool BATCH>
-__global__ void __launch_bounds__(PenGeo::NT, 2) k_godunov_pen(const __grid_constant__ ColArgs a)
+__global__ void __launch_bounds__(PenGeo::NT, 2) k_godunov_pen(ColArgs a)
 {
     using G = PenGeo;
     using S = PenSmem<FINER>;
@@ -499,12 +499,7 @@ amr_status launch_pen(const amr_tree *t, const hydro_params *p, const double *u_
     const size_t bytes = finer ? sizeof(PenSmem<true>) : sizeof(PenSmem<false>);
     auto kern = t->n_inst > 0 ? k_godunov_pen<RS, false, true>
                               : finer ? k_godunov_pen<RS, true, false> : k_godunov_pen<RS, false, false>;
-    AMR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
-    AMR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    a.share = a.zc > 0 ? a.zc : even_share(a.planes, resident_ctas(kern, G::NT, bytes));
-    kern<<<unsigned((a.planes + a.share - 1) / a.share), G::NT, bytes, st>>>(a);
-    AMR_CUDA_TRY(cudaGetLastError());
-    return AMR_OK;
+    return launch_kernel(kern, G::NT, bytes, true, st, a, column_grid);
 }
 
 }  // namespace amr
