@@ -6,6 +6,10 @@
  * neighbours 1/6, Sec. 2.3) and the convergence measure of Eq. 3,
  * eps_i = sqrt((r_i . u_i) / (r_0 . u_0)), u_i = M^-1 r_i.
  *
+ * On one GPU the iteration runs in the single-reduction form the pipelined one is derived
+ * from (Algorithm 2 there): the same iterates in exact arithmetic, without the recurrences
+ * that only hide a distributed reduction.
+ *
  * Linear system: A x = b on a box of nx*ny*nz cells.  Vectors are FP64 arrays of
  * n = nx*ny*nz entries indexed i + nx (j + ny k).  A = 6 I - N with (N v)_c the sum of v
  * over the face neighbours of cell c inside the box: the 7-point Laplacian times -h^2
@@ -45,7 +49,7 @@ typedef struct {
     double tol;               /* stop at the first i >= 1 with eps_i <= tol; >= 0 */
     int32_t max_iter;         /* >= 0 */
     int32_t check_every;      /* ppcg_solve: iterations launched between host checks (0: 16) */
-    int32_t tile_y;           /* rows of the 32-wide tile of one thread block: 8 or 16 (0: 8) */
+    int32_t tile_y;           /* rows of the 32-wide tile of one thread block: 8 or 16 (0: chosen) */
     int32_t seg;              /* z planes one thread block marches through (0: chosen; else >= 4) */
 } ppcg_params;
 
@@ -73,7 +77,7 @@ amr_status ppcg_start(const ppcg_params *prm, const double *d_b, const double *d
                       size_t work_bytes, double *d_eps, amr_stream stream);
 
 /* Launch `count` PPCG iterations, one fused kernel each (both preconditioner and operator
-   applications, the eight vector recurrences and the next iteration's two inner
+   applications, the vector recurrences and the next iteration's two inner
    products; the last thread block to finish reduces the inner products in a fixed order
    and computes the next step length).  Iterations after the solve has stopped return at
    once, so over-launching is harmless.  d_x is updated in place.  Asynchronous. */

@@ -2,27 +2,36 @@
 // Algorithm 4) with the 7-point incomplete-Poisson preconditioner (13/12, 1/6) and the
 // convergence measure of Eq. 3.  FP64 throughout.
 //
-// One iteration is one kernel.  A thread block owns a 32 x TY column of cells and marches
-// up a segment of z planes, keeping rings of w planes (with a two-cell in-plane halo) and
-// of m = M^-1 w planes (one-cell halo) in shared memory, so that m_i = M^-1 w_i and
-// n_i = A m_i never touch HBM.  Each cell then runs the eight recurrences of the
-// iteration (z, q, s, p with beta_i; x, r, u, w with alpha_i) and adds its share of
-// gamma_{i+1} = r_{i+1} . u_{i+1} and delta_{i+1} = w_{i+1} . u_{i+1}.  The last block to
-// finish reduces the per-block partials in a fixed order (so results do not depend on
-// scheduling) and computes eps_{i+1}, beta_{i+1}, alpha_{i+1} for the next launch: the
-// kernel boundary is the iteration's single global synchronisation, the role the
-// all-reduce plays in the distributed algorithm.  w is double-buffered because
-// neighbouring blocks read its halo; every other vector is read and written only at the
-// thread's own cell.
+// One iteration is one kernel, in one of two forms (chosen by plan()).
+//
+// Pipelined (k_iter_pipe), as printed: m = M^-1 w, n = A m, eight recurrences.  A thread block
+// owns a 32 x TY column of cells and marches up a segment of z planes, keeping rings of w planes
+// (two-cell in-plane halo) and of m planes (one-cell halo) in shared memory.  FP64 work 29
+// operations a cell (halo included), 128 bytes.
+//
+// Single-reduction (k_iter; Chronopoulos & Gear 1989; Ghysels & Vanroose 2014, Algorithm 2, from
+// which the pipelined form is derived; the iterates and Eq. 3 are the same in exact arithmetic):
+// s = w + beta s, r = r - alpha s, u = M^-1 r, w = A u, p = u + beta p, x = x + alpha p.  The
+// pipelined recurrences for z = A q, q = M^-1 s and u let a distributed reduction overlap the
+// stencils; here the kernel boundary is the only synchronisation, and they cost FP64 operations
+// (29 a cell against 22, the bound) and traffic (128 bytes against 96).  A block forms r and s of
+// each plane with a two-cell halo (and writes its own cells'), keeps r in a ring of four planes
+// and u (one-cell halo) in a ring of three, and from those u and w.  After 150 iterations x is
+// 2e-15 from the textbook iteration in 64 bits, 1e-12 with the pipelined recurrences.
+//
+// In both, the last block to finish reduces the inner products (r, u), (w, u) of all blocks in a
+// fixed order (so results do not depend on scheduling) and computes eps, beta, alpha for the next
+// launch: the role the all-reduce plays in the distributed algorithm.  Vectors that neighbouring
+// blocks read are double-buffered; every other one is read and written at the thread's own cell.
 //
 // The solver applies 6 M^-1 (centre 6.5, neighbours 1), one FP64 instruction per
 // application fewer than the 13/12, 1/6 stencil.  Scaling the preconditioner by c > 0
 // leaves x_i and eps_i unchanged in exact arithmetic (u, w, gamma scale by c; m, q, n, z,
-// delta by c^2; alpha by 1/c; beta not at all), and FP64 arithmetic is the bound of the
-// iteration kernel on this GPU.
+// delta by c^2; alpha by 1/c; beta not at all), and FP64 arithmetic is the bound of the iteration
+// kernels on this GPU.
 //
-// Without a preconditioner (M^-1 = I) the recurrences give m = w, q = s and u = r
-// exactly, so that variant keeps r, s, w, z, p only and applies A to w directly.
+// Without a preconditioner (M^-1 = I) the recurrences give m = w, q = s and u = r exactly, so that
+// variant of the pipelined kernel keeps r, s, w, z, p only and applies A to w directly.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -50,7 +59,7 @@ struct Dims {
 };
 
 struct Vecs {
-    double *r, *u, *w0, *w1, *z, *q, *s, *p;
+    double *r0, *r1, *u, *w0, *w1, *s0, *s1, *p;
 };
 
 struct Work {
@@ -84,7 +93,7 @@ Work carve(void *base, int nx, int ny, int nz)
     w.part_cap = part_capacity(nx, ny, nz);
     w.part = (double *)p;
     p += align256(2 * w.part_cap * 8);
-    double **v[8] = {&w.v.r, &w.v.u, &w.v.w0, &w.v.w1, &w.v.z, &w.v.q, &w.v.s, &w.v.p};
+    double **v[8] = {&w.v.r0, &w.v.r1, &w.v.u, &w.v.w0, &w.v.w1, &w.v.s0, &w.v.s1, &w.v.p};
     for (int i = 0; i < 8; i++) {
         *v[i] = (double *)p;
         p += align256(n * 8);
@@ -251,8 +260,36 @@ __global__ void __launch_bounds__(INIT_THREADS) k_start(Dims d, const double *__
     }
 }
 
+// gamma_{i+1} = ga, delta_{i+1} = da (thread 0 of the last block): eps_{i+1} (Eq. 3) and the next
+// step length
+__device__ void next_step(PState *st, double *eps, int it, double alpha, double ga, double da)
+{
+    const int i1 = it + 1;
+    st->count = 0;
+    st->it = i1;
+    const double e = sqrt(ga / st->gamma0);
+    st->eps = e;
+    if (eps) eps[i1] = e;
+    if (e <= st->tol) {
+        st->status = AMR_OK;
+        st->done = 1;
+    } else if (i1 >= st->max_iter) {
+        st->done = 1;
+    } else {
+        const double b1 = ga / st->gamma;
+        const double a1 = ga / (da - b1 * ga / alpha);
+        if (!(a1 > 0.0) || !isfinite(a1)) {
+            st->status = AMR_EBREAKDOWN;
+            st->done = 1;
+        }
+        st->beta = b1;
+        st->alpha = a1;
+        st->gamma = ga;
+    }
+}
+
 template <int TY, bool PC>
-struct IterSmem {
+struct PipeSmem {
     static constexpr int H = PC ? 2 : 1;          // in-plane halo of the w tile
     static constexpr int WX = TX + 2 * H, WY = TY + 2 * H;
     static constexpr int MX = TX + 2, MY = TY + 2;
@@ -272,17 +309,19 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// One PPCG iteration (see the file comment).  Grid: (ceil(nx/32), ceil(ny/TY), ceil(nz/seg)).
+// One pipelined iteration: m = M^-1 w and n = A m from a ring of w planes, then the eight
+// recurrences (z, q, s, p with beta; x, r, u, w with alpha).  z and q use the second buffers of r
+// and s.  Grid: (ceil(nx/32), ceil(ny/TY), ceil(nz/seg)).
 // Step k of a block's z march: the copy of w plane k+3 (k+2 without preconditioner) is
 // started and the seven vectors of cell (x, y, k) are loaded before the block waits for
 // w plane k+2 and computes m plane k+1, so both kinds of memory latency overlap the
 // previous plane's arithmetic.
 template <int TY, bool PC>
-__global__ void __launch_bounds__(TX *TY, 1024 / (TX * TY)) k_iter(Dims d, Vecs v, double *__restrict__ x, PState *st,
+__global__ void __launch_bounds__(TX *TY, 1024 / (TX * TY)) k_iter_pipe(Dims d, Vecs v, double *__restrict__ x, PState *st,
                                                                   double *part, double *eps, int seg)
 {
     constexpr int NT = TX * TY;
-    using S = IterSmem<TY, PC>;
+    using S = PipeSmem<TY, PC>;
     constexpr int H = S::H, WX = S::WX, WY = S::WY, MX = S::MX, MY = S::MY, RW = S::RW;
     constexpr int AHEAD = PC ? 3 : 2;             // w plane started at step k: k + AHEAD
     __shared__ S sm;
@@ -343,14 +382,14 @@ __global__ void __launch_bounds__(TX *TY, 1024 / (TX * TY)) k_iter(Dims d, Vecs 
         const int64_t c = gx + d.sy * gy + d.sz * k;
         double rc = 0.0, xc = 0.0, uc = 0.0, zo = 0.0, so = 0.0, po = 0.0, qo = 0.0;
         if (own) {
-            rc = v.r[c];
+            rc = v.r0[c];
             xc = x[c];
             if (PC) uc = v.u[c];
             if (!first) {
-                zo = v.z[c];
-                so = v.s[c];
+                zo = v.r1[c];
+                so = v.s0[c];
                 po = v.p[c];
-                if (PC) qo = v.q[c];
+                if (PC) qo = v.s1[c];
             }
         }
         cp_async_wait<1>();
@@ -389,11 +428,11 @@ __global__ void __launch_bounds__(TX *TY, 1024 / (TX * TY)) k_iter(Dims d, Vecs 
         xc = fma(alpha, pp, xc);
         rc = fma(-alpha, ss, rc);
         const double wn = fma(-alpha, zz, wc);
-        v.z[c] = zz; v.s[c] = ss; v.p[c] = pp;
-        x[c] = xc; v.r[c] = rc; wout[c] = wn;
+        v.r1[c] = zz; v.s0[c] = ss; v.p[c] = pp;
+        x[c] = xc; v.r0[c] = rc; wout[c] = wn;
         if (PC) {
             uc = fma(-alpha, qq, uc);
-            v.q[c] = qq; v.u[c] = uc;
+            v.s1[c] = qq; v.u[c] = uc;
         } else {
             uc = rc;
         }
@@ -403,55 +442,258 @@ __global__ void __launch_bounds__(TX *TY, 1024 / (TX * TY)) k_iter(Dims d, Vecs 
     cp_async_wait<0>();
     const int nb = gridDim.x * gridDim.y * gridDim.z;
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
-    if (grid_sum2<NT>(ga, da, sm.red, part, st, nb, bid)) {
-        // gamma_{i+1}, delta_{i+1}; then eps_{i+1} (Eq. 3) and the next step length
-        const int i1 = it + 1;
-        st->count = 0;
-        st->it = i1;
-        const double e = sqrt(ga / st->gamma0);
-        st->eps = e;
-        if (eps) eps[i1] = e;
-        if (e <= st->tol) {
-            st->status = AMR_OK;
-            st->done = 1;
-        } else if (i1 >= st->max_iter) {
-            st->done = 1;
-        } else {
-            const double b1 = ga / st->gamma;
-            const double a1 = ga / (da - b1 * ga / alpha);
-            if (!(a1 > 0.0) || !isfinite(a1)) {
-                st->status = AMR_EBREAKDOWN;
-                st->done = 1;
-            }
-            st->beta = b1;
-            st->alpha = a1;
-            st->gamma = ga;
+    if (grid_sum2<NT>(ga, da, sm.red, part, st, nb, bid)) next_step(st, eps, it, alpha, ga, da);
+}
+
+template <int TY>
+struct IterSmem {
+    static constexpr int H = 2;                   // in-plane halo of the r planes
+    static constexpr int WX = TX + 2 * H, WY = TY + 2 * H;
+    static constexpr int MX = TX + 2, MY = TY + 2;
+    double r[4][WY * WX];                         // ring, slot = plane & 3
+    double u[3][MY * MX];                         // ring, slot = plane mod 3
+    double red[2 * TX * TY / 32];
+};
+
+// The planes of all columns, one column after the other, in equal shares: block b marches planes
+// [b share, (b + 1) share), a segment per column it meets.  With seg > 0 no segment is longer
+// and a block takes one (columns padded to multiples of seg).
+struct March {
+    int64_t planes, share;
+    int seg, cx;
+};
+
+// One iteration (see the file comment).  Step k of a block's z march: the residual plane k+2, loaded during the step before, is formed, the loads of the next one and of the own cell's vectors
+// are started, then u of plane k+1 and w of plane k.  The places of a thread's elements in the
+// halo planes are worked out once: doing so per plane and element (two divisions each) took 265
+// integer operations a cell.
+template <int TY>
+__global__ void __launch_bounds__(TX *TY, 1024 / (TX * TY)) k_iter(Dims d, Vecs v, double *__restrict__ x, PState *st,
+                                                                  double *part, double *eps, March mc)
+{
+    constexpr int NT = TX * TY;
+    using S = IterSmem<TY>;
+    constexpr int H = S::H, WX = S::WX, WY = S::WY, MX = S::MX, MY = S::MY;
+    constexpr int AHEAD = 2;                      // residual plane formed at step k: k + AHEAD
+    constexpr int NE = WX * WY, ER = (NE + NT - 1) / NT;                 // residual elements, per thread
+    constexpr int NU = MX * MY, EU = (NU + NT - 1) / NT;        // u elements, per thread
+    __shared__ S sm;
+    if (st->done) return;
+    const int it = st->it;
+    const double alpha = st->alpha, beta = st->beta;
+    const bool first = it == 0;
+    const bool odd = it & 1;
+    const double *__restrict__ rin = odd ? v.r1 : v.r0, *__restrict__ sin = odd ? v.s1 : v.s0,
+                 *__restrict__ win = odd ? v.w1 : v.w0;
+    double *__restrict__ rout = odd ? v.r0 : v.r1, *__restrict__ sout = odd ? v.s0 : v.s1,
+           *__restrict__ wout = odd ? v.w0 : v.w1;
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    double ga = 0.0, da = 0.0;
+    const int pitch = mc.seg > 0 ? (d.nz + mc.seg - 1) / mc.seg * mc.seg : d.nz;
+    const int64_t gend = min((blockIdx.x + int64_t(1)) * mc.share, mc.planes);
+    for (int64_t g = blockIdx.x * mc.share; g < gend;) {
+        const int64_t col = g / pitch;
+        const int x0 = int(col % mc.cx) * TX, y0 = int(col / mc.cx) * TY;
+        const int z0 = int(g - col * pitch), z1 = int(min(z0 + (gend - g), int64_t(d.nz)));
+        g = mc.seg > 0 ? gend : g + (z1 - z0);
+        const int gx = x0 + tx, gy = y0 + ty;
+        const bool own = gx < d.nx && gy < d.ny;
+        const int64_t oc = gx + d.sy * gy;
+
+        // residual elements e = tid + NT j of a halo plane: offset in the plane, whether inside the
+        // box, whether one of the block's own cells
+        int64_t eo[ER];
+        bool ein[ER], eown[ER];
+#pragma unroll
+        for (int j = 0; j < ER; ++j) {
+            const int e = tid + NT * j, ex = e % WX, ey = e / WX, ix = x0 - H + ex, iy = y0 - H + ey;
+            ein[j] = e < NE && ix >= 0 && ix < d.nx && iy >= 0 && iy < d.ny;
+            eown[j] = ein[j] && ex >= H && ex < H + TX && ey >= H && ey < H + TY;
+            eo[j] = ein[j] ? ix + d.sy * iy : 0;
         }
+        struct Raw {
+            double r[ER], s[ER], w[ER];
+        };
+        auto load = [&](int k, Raw &l) {
+            const int64_t o = d.sz * k;
+            const bool zin = k >= 0 && k < d.nz;
+#pragma unroll
+            for (int j = 0; j < ER; ++j)
+                if (zin && ein[j]) {
+                    l.r[j] = rin[eo[j] + o];
+                    l.w[j] = win[eo[j] + o];
+                    if (!first) l.s[j] = sin[eo[j] + o];
+                }
+        };
+        // r and s of plane k from the loaded values (zero outside the box)
+        auto form = [&](int k, const Raw &l) {
+            const bool zin = k >= 0 && k < d.nz, zown = k >= z0 && k < z1;
+            double *dst = sm.r[k & 3];
+#pragma unroll
+            for (int j = 0; j < ER; ++j) {
+                double rn = 0.0;
+                if (zin && ein[j]) {
+                    const double sn = first ? l.w[j] : fma(beta, l.s[j], l.w[j]);
+                    rn = fma(-alpha, sn, l.r[j]);
+                    if (zown && eown[j]) {
+                        sout[eo[j] + d.sz * k] = sn;
+                        rout[eo[j] + d.sz * k] = rn;
+                    }
+                }
+                if (tid + NT * j < NE) dst[tid + NT * j] = rn;
+            }
+        };
+        // u = 6 M^-1 r on plane k with a one-cell halo (zero outside the box)
+        int ur[EU];
+        bool uin[EU];
+#pragma unroll
+        for (int j = 0; j < EU; ++j) {
+            const int e = tid + NT * j, ex = e % MX, ey = e / MX, ix = x0 - 1 + ex, iy = y0 - 1 + ey;
+            uin[j] = e < NU && ix >= 0 && ix < d.nx && iy >= 0 && iy < d.ny;
+            ur[j] = (ey + 1) * WX + ex + 1;
+        }
+        auto form_u = [&](int k) {
+            double *dst = sm.u[(k + 3) % 3];
+            const double *rm = sm.r[(k - 1) & 3], *rc = sm.r[k & 3], *rp = sm.r[(k + 1) & 3];
+            const bool zin = k >= 0 && k < d.nz;
+#pragma unroll
+            for (int j = 0; j < EU; ++j) {
+                double val = 0.0;
+                if (zin && uin[j]) {
+                    const int i = ur[j];
+                    const double s = ((rc[i - 1] + rc[i + 1]) + (rc[i - WX] + rc[i + WX])) + (rm[i] + rp[i]);
+                    val = fma(6.5, rc[i], s);
+                }
+                if (tid + NT * j < NU) dst[tid + NT * j] = val;
+            }
+        };
+
+        // the first planes, two in flight at a time
+        Raw l, l2;
+        static_assert((H + AHEAD) % 2 == 0, "planes in pairs");
+#pragma unroll
+        for (int k = 0; k < H + AHEAD; k += 2) {
+            load(z0 - H + k, l);
+            load(z0 - H + k + 1, l2);
+            form(z0 - H + k, l);
+            form(z0 - H + k + 1, l2);
+        }
+        load(z0 + AHEAD, l);
+        __syncthreads();
+        form_u(z0 - 1);
+        form_u(z0);
+        __syncthreads();                              // before the first plane is formed over z0 - 2
+        for (int k = z0; k < z1; k++) {
+            form(k + AHEAD, l);
+            if (k + 1 < z1) load(k + AHEAD + 1, l);
+            const int64_t c = oc + d.sz * k;
+            double xc = 0.0, uo = 0.0, po = 0.0;
+            if (own) {
+                xc = x[c];
+                uo = v.u[c];
+                if (!first) po = v.p[c];
+            }
+            __syncthreads();
+            form_u(k + 1);
+            __syncthreads();
+            if (!own) continue;
+            const double *rk = sm.r[k & 3];
+            const int ri = (ty + H) * WX + tx + H;
+            const double rc = rk[ri];
+            const double *uk = sm.u[k % 3], *um = sm.u[(k + 2) % 3], *up = sm.u[(k + 1) % 3];
+            const int mi = (ty + 1) * MX + tx + 1;
+            const double un = uk[mi];
+            const double s = ((uk[mi - 1] + uk[mi + 1]) + (uk[mi - MX] + uk[mi + MX])) + (um[mi] + up[mi]);
+            const double wn = fma(6.0, un, -s);
+            const double pp = first ? uo : fma(beta, po, uo);
+            x[c] = fma(alpha, pp, xc);
+            v.p[c] = pp;
+            wout[c] = wn;
+            v.u[c] = un;
+            ga = fma(rc, un, ga);
+            da = fma(wn, un, da);
+        }
+        __syncthreads();                          // the next segment reuses the rings
     }
+    if (grid_sum2<NT>(ga, da, sm.red, part, st, gridDim.x, blockIdx.x)) next_step(st, eps, it, alpha, ga, da);
 }
 
 struct Launch {
     dim3 grid;
-    int ty, seg;
+    int ty;
+    bool pipe;       // the pipelined kernel (else the single-reduction one)
+    int seg;
+    March mc;
 };
+
+// Which kernel, tile height and split of the z planes.  Single-reduction form: with the
+// preconditioner, on boxes of at least SINGLE_CELLS cells.  Per iteration, pipelined against
+// single-reduction: 64^3 30.9 / 32.8 us, 180 x 141 x 117 187 / 164, 256^3 825 / 740; without
+// preconditioner the forms take the same FP64 work, and the pipelined one needs one halo instead
+// of three: 64^3 20.9 / 22.6, 256^3 483 / 472.
+constexpr int64_t SINGLE_CELLS = 700000;
 
 amr_status plan(const ppcg_params *prm, Launch &L)
 {
-    L.ty = prm->tile_y ? prm->tile_y : 8;
-    if (L.ty != 8 && L.ty != 16) return AMR_EINVAL;
-    const int cx = (prm->nx + TX - 1) / TX, cy = (prm->ny + L.ty - 1) / L.ty;
+    const int nx = prm->nx, ny = prm->ny, nz = prm->nz, cx = (nx + TX - 1) / TX;
     int seg = prm->seg;
-    if (seg == 0) {
-        const int64_t cols = (int64_t)cx * cy;
-        int64_t nseg = (INIT_BLOCKS + cols - 1) / cols;
-        seg = (int)((prm->nz + nseg - 1) / nseg);
-        if (seg < MIN_SEG) seg = MIN_SEG;
+    if (prm->tile_y != 0 && prm->tile_y != 8 && prm->tile_y != 16) return AMR_EINVAL;
+    if (seg != 0 && seg < MIN_SEG) return AMR_EINVAL;
+    L.pipe = prm->precond != PPCG_PRECOND_IP || (int64_t)nx * ny * nz < SINGLE_CELLS;
+    // 16 rows repeat less of the halo in the single-reduction form (20 instead of 22 FP64
+    // operations a cell): 256^3 715 us an iteration against 757, 180 x 141 x 117 164 against 168
+    L.ty = prm->tile_y ? prm->tile_y : L.pipe ? 8 : 16;
+    const int cy = (ny + L.ty - 1) / L.ty;
+    const int64_t cols = (int64_t)cx * cy;
+    if (cy > 65535 || (seg > 0 && (nz + seg - 1) / seg > 65535)) return AMR_EINVAL;
+    if (L.pipe) {
+        if (seg == 0) {
+            int64_t nseg = (INIT_BLOCKS + cols - 1) / cols;
+            seg = (int)((nz + nseg - 1) / nseg);
+            if (seg < MIN_SEG) seg = MIN_SEG;
+        }
+        const int cz = (nz + seg - 1) / seg;
+        if (cz > 65535) return AMR_EINVAL;
+        L.seg = seg;
+        L.grid = dim3(cx, cy, cz);
+        return AMR_OK;
     }
-    if (seg < MIN_SEG) return AMR_EINVAL;
-    const int cz = (prm->nz + seg - 1) / seg;
-    if (cy > 65535 || cz > 65535) return AMR_EINVAL;
-    L.seg = seg;
-    L.grid = dim3(cx, cy, cz);
+    int dev = 0, nsm = 152;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int64_t slots = (int64_t)nsm * (1024 / (TX * L.ty));
+    L.mc.cx = cx;
+    L.mc.seg = seg;
+    if (seg == 0) {
+        // Segments of one length: the one with the shortest estimated time, whole waves of
+        // resident blocks, each its planes plus about three planes' worth of halo.  Where that
+        // leaves the last wave half empty, equal shares of all planes in one wave instead
+        // (180 x 141 x 117: 164 us an iteration against 170).  Not otherwise: neighbouring columns
+        // are then at different heights and re-read each other's halo from memory.
+        int64_t best = -1;
+        for (int nseg = 1; nseg <= 64 && nseg <= nz; nseg++) {
+            int s = (nz + nseg - 1) / nseg;
+            if (s < MIN_SEG) s = MIN_SEG;
+            const int64_t blocks = cols * ((nz + s - 1) / s);
+            const int64_t cost = ((blocks + slots - 1) / slots) * (s + 3);
+            if (best < 0 || cost < best) {
+                best = cost;
+                L.mc.seg = s;
+            }
+        }
+        const int64_t share = (cols * nz + slots - 1) / slots;
+        if (share >= 12 && double(share) + 2.5 * (1.0 + double(share) / nz) < 0.9 * double(best)) {
+            L.mc.seg = 0;
+            L.mc.share = share;
+            L.mc.planes = cols * nz;
+        }
+    }
+    if (L.mc.seg > 0) {
+        L.mc.share = L.mc.seg;
+        L.mc.planes = cols * ((nz + L.mc.seg - 1) / L.mc.seg) * L.mc.seg;
+    }
+    const int64_t blocks = (L.mc.planes + L.mc.share - 1) / L.mc.share;
+    if (blocks > INT32_MAX) return AMR_EINVAL;
+    L.grid = dim3((unsigned)blocks);
     return AMR_OK;
 }
 
@@ -518,12 +760,12 @@ extern "C" amr_status ppcg_start(const ppcg_params *prm, const double *d_b, cons
     Work w = carve(d_work, prm->nx, prm->ny, prm->nz);
     if (cudaMemsetAsync(w.st, 0, sizeof(PState), st) != cudaSuccess) return AMR_ECUDA;
     const int g = init_grid(d.n);
-    k_resid<<<g, INIT_THREADS, 0, st>>>(d, d_b, d_x, w.v.r);
+    k_resid<<<g, INIT_THREADS, 0, st>>>(d, d_b, d_x, w.v.r0);
     if (prm->precond == PPCG_PRECOND_IP)
-        k_start<true><<<g, INIT_THREADS, 0, st>>>(d, w.v.r, w.v.u, w.v.w0, w.st, w.part, d_eps, prm->tol,
+        k_start<true><<<g, INIT_THREADS, 0, st>>>(d, w.v.r0, w.v.u, w.v.w0, w.st, w.part, d_eps, prm->tol,
                                                     prm->max_iter);
     else
-        k_start<false><<<g, INIT_THREADS, 0, st>>>(d, w.v.r, w.v.u, w.v.w0, w.st, w.part, d_eps, prm->tol,
+        k_start<false><<<g, INIT_THREADS, 0, st>>>(d, w.v.r0, w.v.u, w.v.w0, w.st, w.part, d_eps, prm->tol,
                                                      prm->max_iter);
     return cuda_status(cudaGetLastError());
 }
@@ -540,13 +782,17 @@ extern "C" amr_status ppcg_iterate(const ppcg_params *prm, double *d_x, void *d_
     Dims d = dims_of(prm->nx, prm->ny, prm->nz);
     Work w = carve(d_work, prm->nx, prm->ny, prm->nz);
     const bool pc = prm->precond == PPCG_PRECOND_IP;
+    const int nt = TX * L.ty;
     for (int i = 0; i < count; i++) {
-        if (L.ty == 16) {
-            if (pc) k_iter<16, true><<<L.grid, TX * 16, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.seg);
-            else k_iter<16, false><<<L.grid, TX * 16, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.seg);
+        if (!L.pipe) {
+            if (L.ty == 16) k_iter<16><<<L.grid, nt, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.mc);
+            else k_iter<8><<<L.grid, nt, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.mc);
+        } else if (L.ty == 16) {
+            if (pc) k_iter_pipe<16, true><<<L.grid, nt, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.seg);
+            else k_iter_pipe<16, false><<<L.grid, nt, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.seg);
         } else {
-            if (pc) k_iter<8, true><<<L.grid, TX * 8, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.seg);
-            else k_iter<8, false><<<L.grid, TX * 8, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.seg);
+            if (pc) k_iter_pipe<8, true><<<L.grid, nt, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.seg);
+            else k_iter_pipe<8, false><<<L.grid, nt, 0, st>>>(d, w.v, d_x, w.st, w.part, d_eps, L.seg);
         }
     }
     return cuda_status(cudaGetLastError());
