@@ -123,24 +123,99 @@ template <> struct Lay<3> { static constexpr int MT = 4, NT = 9, K = H, OW = OW3
 template <> struct Lay<4> { static constexpr int MT = 1, NT = 9, K = H, OW = OW4, OB = OB4, NOUTS = NOUT; };
 template <int L> __host__ __device__ constexpr int slots() { return (Lay<L>::MT * Lay<L>::NT + 7) / 8; }
 
+// 8 x 8 BF16 blocks of shared memory as MMA fragments (ldmatrix), and fragments stored as
+// transposed blocks (stmatrix .trans): one instruction for what took four to sixteen loads or
+// stores of 2 or 4 bytes, which were a third of a training step's instructions.
+__device__ __forceinline__ unsigned saddr(const void *p) { return unsigned(__cvta_generic_to_shared(p)); }
+__device__ __forceinline__ void ldm4(uint32_t r[4], unsigned addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ void stm4t(unsigned addr, const uint32_t r[4])
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(r[0]), "r"(r[1]),
+                 "r"(r[2]), "r"(r[3])
+                 : "memory");
+}
+// B fragments of n-tile nt, k-tiles kt and kt + 1, of a row-major [N][stride] block
+__device__ __forceinline__ void bfrag2(const __nv_bfloat16 *W, int stride, int nt, int kt, int lane, uint32_t b[4])
+{
+    ldm4(b, saddr(W + (nt * 8 + (lane & 7)) * stride + kt * 16 + (lane >> 3) * 8));
+}
+// B fragments of n-tiles nt and nt + 1, k-tile 0
+__device__ __forceinline__ void bfrag2n(const __nv_bfloat16 *W, int stride, int nt, int lane, uint32_t b[4])
+{
+    ldm4(b, saddr(W + ((nt + (lane >> 4)) * 8 + (lane & 7)) * stride + ((lane >> 3) & 1) * 8));
+}
+
+// the forward pass of 16 samples with the weights in shared memory (forward16's arithmetic in its
+// order); keeps the pre-activations of the hidden layers
+__device__ __forceinline__ void forward16_sm(const Packed &P, const float *x16, int lane, float out[4], float (*z)[8][4])
+{
+    uint32_t a0[4], a[4][4], b[4];
+    input_frag(x16, lane, a0);
+    bias_init(z[0], P.b, lane);
+#pragma unroll
+    for (int nt = 0; nt < 8; nt += 2) {
+        bfrag2n(P.w + PW1, S1, nt, lane, b);
+        mma16816(z[0][nt], a0, b[0], b[1]);
+        mma16816(z[0][nt + 1], a0, b[2], b[3]);
+    }
+#pragma unroll
+    for (int layer = 0; layer < 2; ++layer) {
+        acc_to_a_silu(z[layer], a);
+        const __nv_bfloat16 *W = P.w + (layer == 0 ? PW2 : PW3);
+        bias_init(z[layer + 1], P.b + H * (layer + 1), lane);
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+            for (int kt = 0; kt < 4; kt += 2) {
+                bfrag2(W, S, nt, kt, lane, b);
+                mma16816(z[layer + 1][nt], a[kt], b[0], b[1]);
+                mma16816(z[layer + 1][nt], a[kt + 1], b[2], b[3]);
+            }
+    }
+    acc_to_a_silu(z[2], a);
+    const int t = lane & 3;
+    float o[4] = {P.b[3 * H + 2 * t], P.b[3 * H + 2 * t + 1], P.b[3 * H + 2 * t], P.b[3 * H + 2 * t + 1]};
+#pragma unroll
+    for (int kt = 0; kt < 4; kt += 2) {
+        bfrag2(P.w + PW4, S, 0, kt, lane, b);
+        mma16816(o, a[kt], b[0], b[1]);
+        mma16816(o, a[kt + 1], b[2], b[3]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) out[i] = o[i];
+}
+
+// stage the BF16 fragments of a [16 samples][64] block of warp w as transposed rows
+__device__ __forceinline__ void stage_T(__nv_bfloat16 (*dst)[TS], const uint32_t a[4][4], int w, int lane)
+{
+#pragma unroll
+    for (int kt = 0; kt < 4; ++kt)
+        stm4t(saddr(&dst[kt * 16 + (lane >> 4) * 8 + (lane & 7)][16 * w + ((lane >> 3) & 1) * 8]), a[kt]);
+}
+
 template <int L>
 __device__ __forceinline__ void grad_gemm(const TrainSmem &sm, float acc[][4], int w, int lane)
 {
     using Y = Lay<L>;
-    const int g = lane >> 2, t = lane & 3;
 #pragma unroll
     for (int sl = 0; sl < slots<L>(); ++sl) {
         const int j = w + 8 * sl;
         if (j >= Y::MT * Y::NT) break;
         const int mt = j / Y::NT, nt = j % Y::NT;
 #pragma unroll
-        for (int kt = 0; kt < TB / 16; ++kt) {
-            uint32_t a[4];
-            const __nv_bfloat16 *A0 = &sm.dzT[mt * 16 + g][kt * 16 + 2 * t];
-            const __nv_bfloat16 *A1 = &sm.dzT[mt * 16 + g + 8][kt * 16 + 2 * t];
-            a[0] = ld32(A0); a[1] = ld32(A1); a[2] = ld32(A0 + 8); a[3] = ld32(A1 + 8);
-            const __nv_bfloat16 *B = &sm.aT[nt * 8 + g][kt * 16 + 2 * t];
-            mma16816(acc[sl], a, ld32(B), ld32(B + 8));
+        for (int kt = 0; kt < TB / 16; kt += 2) {
+            uint32_t b[4], a[4];
+            ldm4(b, saddr(&sm.aT[nt * 8 + (lane & 7)][kt * 16 + (lane >> 3) * 8]));
+            ldm4(a, saddr(&sm.dzT[mt * 16 + (lane & 15)][kt * 16 + (lane >> 4) * 8]));
+            mma16816(acc[sl], a, b[0], b[1]);
+            ldm4(a, saddr(&sm.dzT[mt * 16 + (lane & 15)][(kt + 1) * 16 + (lane >> 4) * 8]));
+            mma16816(acc[sl], a, b[2], b[3]);
         }
     }
 }
@@ -167,36 +242,6 @@ __device__ __forceinline__ void grad_store(const float acc[][4], float *out, int
             else if (k == kones) out[Y::OB + n] = acc[sl][i];
         }
     }
-}
-
-// stage the BF16 SiLU activations (as the forward pass computes them) transposed
-__device__ __forceinline__ void stage_T_silu(__nv_bfloat16 (*dst)[TS], const float v[8][4], int w, int lane)
-{
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t p = silu_bf16x2(v[nt][2 * h], v[nt][2 * h + 1]);
-            const int row = 16 * w + g + (h ? 8 : 0);
-            const int col = nt * 8 + 2 * t;
-            dst[col][row] = *reinterpret_cast<const __nv_bfloat16 *>(&p);
-            dst[col + 1][row] = *(reinterpret_cast<const __nv_bfloat16 *>(&p) + 1);
-        }
-}
-
-// stage an accumulator-layout [16 samples][64] block of warp w as bf16 transposed rows
-template <typename F>
-__device__ __forceinline__ void stage_T(__nv_bfloat16 (*dst)[TS], const float v[8][4], int w, int lane, F f)
-{
-    const int g = lane >> 2, t = lane & 3;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int col = nt * 8 + 2 * t + (i & 1), row = 16 * w + g + (i >= 2 ? 8 : 0);
-            dst[col][row] = __float2bfloat16_rn(f(v[nt][i]));
-        }
 }
 
 // mode 0: loss = sum over samples and outputs of (y - target)^2 / n, dy = 2 (y - t) / n
@@ -241,7 +286,7 @@ __global__ void __launch_bounds__(256, 1) k_train_grad(const void *packed, const
         }
         __syncwarp();
         float z[3][8][4], o[4];
-        forward16(P, sm.sx[w], lane, o, z);
+        forward16_sm(P, sm.sx[w], lane, o, z);
         // dy in the output-fragment layout (lanes t == 0 own outputs 0, 1)
         float dz4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         if (t == 0) {
@@ -261,6 +306,7 @@ __global__ void __launch_bounds__(256, 1) k_train_grad(const void *packed, const
         }
         // ---- layer 4: dW4 = dz4^T a3, da3 = dz4 W4
         float v8[8][4];
+        uint32_t a[4][4], b[4];
         __syncthreads();   // previous chunk's gradient products are done with the buffers
         // rows 0..15 of dz^T for this warp's 16 sample columns: outputs 0, 1 and zero padding
         for (int j = lane; j < 16 * 16; j += 32) sm.dzT[j / 16][16 * w + (j % 16)] = __float2bfloat16_rn(0.0f);
@@ -269,20 +315,22 @@ __global__ void __launch_bounds__(256, 1) k_train_grad(const void *packed, const
 #pragma unroll
             for (int i = 0; i < 4; ++i) sm.dzT[i & 1][16 * w + g + (i >= 2 ? 8 : 0)] = __float2bfloat16_rn(dz4[i]);
         }
-        stage_T_silu(sm.aT, z[2], w, lane);
+        acc_to_a_silu(z[2], a);
+        stage_T(sm.aT, a, w, lane);
         __syncthreads();
         grad_gemm<4>(sm, g4, w, lane);
         {
-            uint32_t a[4];
-            a[0] = pack_bf16(dz4[0], dz4[1]);
-            a[1] = pack_bf16(dz4[2], dz4[3]);
-            a[2] = 0u; a[3] = 0u;
+            uint32_t d4[4];
+            d4[0] = pack_bf16(dz4[0], dz4[1]);
+            d4[1] = pack_bf16(dz4[2], dz4[3]);
+            d4[2] = 0u; d4[3] = 0u;
 #pragma unroll
-            for (int nt = 0; nt < 8; ++nt) {
+            for (int nt = 0; nt < 8; nt += 2) {
                 v8[nt][0] = v8[nt][1] = v8[nt][2] = v8[nt][3] = 0.0f;
-                uint32_t b0, b1;
-                bfrag(P.w + PW4T, S4T, nt, 0, lane, b0, b1);
-                mma16816(v8[nt], a, b0, b1);
+                v8[nt + 1][0] = v8[nt + 1][1] = v8[nt + 1][2] = v8[nt + 1][3] = 0.0f;
+                bfrag2n(P.w + PW4T, S4T, nt, lane, b);
+                mma16816(v8[nt], d4, b[0], b[1]);
+                mma16816(v8[nt + 1], d4, b[2], b[3]);
             }
         }
         // ---- layers 3, 2: dz = da * silu'(z); dW = dz^T a_prev; da_prev = dz W
@@ -293,23 +341,24 @@ __global__ void __launch_bounds__(256, 1) k_train_grad(const void *packed, const
             for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) v8[nt][i] *= dsilu(zl[nt][i]);
+            uint32_t dz[4][4];
+            acc_to_a(v8, dz, [](float q) { return q; });
+            acc_to_a_silu(z[L - 2], a);
             __syncthreads();
-            stage_T(sm.dzT, v8, w, lane, [](float q) { return q; });
-            stage_T_silu(sm.aT, z[L - 2], w, lane);
+            stage_T(sm.dzT, dz, w, lane);
+            stage_T(sm.aT, a, w, lane);
             __syncthreads();
             if (L == 3) grad_gemm<3>(sm, g3, w, lane);
             else grad_gemm<2>(sm, g2, w, lane);
-            uint32_t a[4][4];
-            acc_to_a(v8, a, [](float q) { return q; });
             const __nv_bfloat16 *WT = P.w + (L == 3 ? PW3T : PW2T);
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
                 v8[nt][0] = v8[nt][1] = v8[nt][2] = v8[nt][3] = 0.0f;
 #pragma unroll
-                for (int kt = 0; kt < 4; ++kt) {
-                    uint32_t b0, b1;
-                    bfrag(WT, S, nt, kt, lane, b0, b1);
-                    mma16816(v8[nt], a[kt], b0, b1);
+                for (int kt = 0; kt < 4; kt += 2) {
+                    bfrag2(WT, S, nt, kt, lane, b);
+                    mma16816(v8[nt], dz[kt], b[0], b[1]);
+                    mma16816(v8[nt], dz[kt + 1], b[2], b[3]);
                 }
             }
         }
@@ -318,8 +367,9 @@ __global__ void __launch_bounds__(256, 1) k_train_grad(const void *packed, const
         for (int nt = 0; nt < 8; ++nt)
 #pragma unroll
             for (int i = 0; i < 4; ++i) v8[nt][i] *= dsilu(z[0][nt][i]);
+        acc_to_a(v8, a, [](float q) { return q; });
         __syncthreads();
-        stage_T(sm.dzT, v8, w, lane, [](float q) { return q; });
+        stage_T(sm.dzT, a, w, lane);
         for (int j = lane; j < 16 * 16; j += 32) {
             const int row = j / 16, k = j % 16;     // sample row, input k
             float v = 0.0f;
