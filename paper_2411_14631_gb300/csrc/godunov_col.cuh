@@ -42,6 +42,7 @@ template <typename R, int FX, int FY, bool FINER> struct ColSmem {
     // refined flag of each stencil cell, slot = plane & 7 (live: k-1 .. k+5, longer than the
     // W ring); only when the level has finer levels
     uint8_t ref[FINER ? 8 : 1][FINER ? SY * SX : 1];
+    float best_dt;                                   // smallest CFL candidate of the segment so far (FP64)
 };
 
 struct ColArgs {
@@ -399,11 +400,13 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
                 sk[0] = rp[si - 1]; sk[1] = rp[si + 1]; sk[2] = rp[si - SX]; sk[3] = rp[si + SX];
                 sk[4] = sm.ref[(p - 1) & 7][si]; sk[5] = sm.ref[(p + 1) & 7][si];
             }
-            R dU[NV] = {0, 0, 0, 0, 0};
+            R dU[NV];
             const int fzl = q3(p), fzu = fzl == 2 ? 0 : fzl + 1;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                if (!sk[0]) dU[v] = dU[v] + sm.Fx[dz][v][x ? x - 1 + FX * y : FX * FY + y];
+                dU[v] = R(0);
+                // the first flux is taken, not added to zero (an FP64 operation)
+                if (!sk[0]) dU[v] = sm.Fx[dz][v][x ? x - 1 + FX * y : FX * FY + y];
                 if (!sk[1]) dU[v] = dU[v] - sm.Fx[dz][v][x + FX * y];
                 if (!sk[2]) dU[v] = dU[v] + sm.Fy[dz][v][x + FX * y];
                 if (!sk[3]) dU[v] = dU[v] - sm.Fy[dz][v][x + FX * (y + 1)];
@@ -421,7 +424,18 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
             }
             if (!state_finite<R>(Un)) set_error(a.status, AMR_ENONPHYSICAL);
             if (uc == 0) sm.cell0[ub][uo8] = cid;
-            if (dtn && !nbref) my_dt = min(my_dt, (unsigned long long)__double_as_longlong(cfl_candidate<R>(Un, pr, cflR, dxR)));
+            if constexpr (sizeof(R) == 8) {
+                if (dtn && !nbref && !cfl_above(Un, pr, cflR, dxR, *const_cast<volatile float *>(&sm.best_dt))) {
+                    const double cand = cfl_candidate<R>(Un, pr, cflR, dxR);
+                    my_dt = min(my_dt, (unsigned long long)__double_as_longlong(cand));
+                    // positive floats compare as their bits; a candidate that is not finite or not
+                    // positive leaves the best as it is
+                    const float cf = d2f_bits(cand);
+                    if (cf > 0.0f) atomicMin(reinterpret_cast<int *>(&sm.best_dt), __float_as_int(cf));
+                }
+            } else if (dtn && !nbref) {
+                my_dt = min(my_dt, (unsigned long long)__double_as_longlong(cfl_candidate<R>(Un, pr, cflR, dxR)));
+            }
         };
         // restriction of the father of one oct of slab k (its eight cells in order), variable v
         auto restrict_one = [&](int k, int w) {
@@ -441,6 +455,7 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
         // predictions z0-1, z0, the z face below z0 together with planes z0+2, z0+3 (which
         // replace the dead z0-2, z0-1), predictions z0+1, z0+2 (replacing z0-1), the faces
         // of slab z0; first the oct tables of layers z0/2-1 .. z0/2+2
+        if (tid == 0) sm.best_dt = __int_as_float(0x7F800000);
         for (int w = tid; w < 4 * NO; w += nt) oct_fill(z0 / 2 - 1 + w / NO, w % NO);
         __syncthreads();
         gather(z0 / 2 - 1);

@@ -206,6 +206,7 @@ struct Smem {
     uint8_t gfull[G::NFULL];
     uint16_t gedge[2 * G::NEDGE];
     std::conditional_t<(G::NP < 256), uint8_t, uint16_t> plist[G::NPN];
+    uint8_t outside[3];             // per tile (index modulo 3): whether a slot lies beyond an outflow face
 };
 static_assert(Geo<2>::NSLOT <= 256, "slot indices fit a byte");
 
@@ -413,6 +414,7 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
     unsigned n_acc = 0, n_fb = 0;   // surrogate: accepted faces, fallbacks (counted by lane 0)
     unsigned n_it = 0, n_solve = 0; // Newton iterations and Newton solves of this thread
     unsigned long long my_dt = ~0ull;   // bit pattern of the smallest positive CFL candidate
+    float best_dt = __int_as_float(0x7F800000);   // the same in FP32 (FP64 path; see cfl_above)
     auto flush_dt = [&](double *target, unsigned long long m) {
         if (!target) return;
         for (int off = 16; off > 0; off >>= 1) m = umin64(m, __shfl_xor_sync(0xffffffffu, m, off));
@@ -467,7 +469,10 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
             }
         }
     }
-    for (int64_t t = a.t_begin + blockIdx.x; t < a.t_end; t += gridDim.x) {
+    if (tid < 3) sm.outside[tid] = 0;
+    __syncthreads();
+    int turn = 0;                   // tiles so far, modulo 3
+    for (int64_t t = a.t_begin + blockIdx.x; t < a.t_end; t += gridDim.x, turn = turn == 2 ? 0 : turn + 1) {
         // ---- level of this tile and its geometry
         const int32_t root = a.tile_root[t];
         int l = a.lfirst;
@@ -495,7 +500,7 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
             lam = scale_pow2(*a.dt, l);    // dt / dx, exact
             dtn = a.dt_next;
         }
-        int mine_out = 0;
+        int mine_upd = 0;            // this thread's slot is an updated oct with a leaf cell
         const bool finer = !a.tile_inst && l < tv.levelmax;   // only then can a stencil cell be refined
         if (tid < G::NSLOT) {
             int32_t e;
@@ -508,14 +513,27 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
                 rf = e >= 0 ? tv.refmask[e] : 0;
             }
             sm.slot[tid] = e;
-            sm.ref[tid] = (e >= 0 && finer) ? rf : 0;
-            mine_out = (e == OUTSIDE);
+            rf = (e >= 0 && finer) ? rf : 0;
+            sm.ref[tid] = rf;
+            if (e == OUTSIDE) sm.outside[turn] = 1;
+            const int sx = tid % G::NS, sy = (tid / G::NS) % G::NS, sz = tid / (G::NS * G::NS);
+            mine_upd = e >= 0 && rf != 0xFF && sx > 0 && sx < G::NS - 1 && sy > 0 && sy < G::NS - 1 && sz > 0 &&
+                       sz < G::NS - 1;
         }
-        const int any_outside = __syncthreads_or(mine_out);   // barrier: slots visible to all
+        // the flag of the next tile, last read two barriers ago
+        if (tid == 0) sm.outside[turn == 2 ? 0 : turn + 1] = 0;
+        const int any_updated = __syncthreads_or(mine_upd);   // barrier: slots visible to all
+        const int any_outside = sm.outside[turn];
         // the next tile's slot entries (their refinement masks after the predictor)
         const int64_t t_nx = t + gridDim.x;
         have_nx = t_nx < a.t_end;
         if (have_nx && tid < G::NSLOT) e_nx = a.tile_slot[t_nx * G::NSLOT + tid];
+        // every cell refined (the middle of a finer level): nothing of this tile is updated, and
+        // no face of it is used
+        if (!any_updated && !a.harvest) {
+            if (have_nx && tid < G::NSLOT) rf_nx = e_nx >= 0 ? tv.refmask[e_nx] : 0;
+            continue;
+        }
 
         // ---- phase 1: gather + primitives of the listed cells (c fastest so a warp reads
         // whole octs)
@@ -694,7 +712,9 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
             if ((sm.ref[s] >> c) & 1) continue;   // refined: its value comes from the restriction
             const int cx = c & 1, cy = (c >> 1) & 1, cz = (c >> 2) & 1;
             const int ii[3] = {2 * ox + cx - 2, 2 * oy + cy - 2, 2 * oz + cz - 2};   // interior coords 0..CI-1
-            R dU[NV] = {0, 0, 0, 0, 0};     // flux sums in the working precision
+            R dU[NV];                       // flux sums in the working precision
+#pragma unroll
+            for (int v = 0; v < NV; ++v) dU[v] = R(0);
             bool nbref = false;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
@@ -712,7 +732,9 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
 #pragma unroll
                     for (int v = 0; v < NV; ++v) {
                         const R F = sF[d][v][r0];
-                        dU[v] = side ? dU[v] - F : dU[v] + F;
+                        // the first flux is taken, not added to zero (an FP64 operation)
+                        if (d == 0 && side == 0) dU[v] = F;
+                        else dU[v] = side ? dU[v] - F : dU[v] + F;
                     }
                 }
             }
@@ -732,13 +754,23 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
             if (!state_finite<R>(Un)) set_error(a.status, AMR_ENONPHYSICAL);
             if (dtn && !nbref) {
                 // CFL candidate (newdt_fine) from the final new state of this leaf cell
-                const double cand = cfl_candidate<R>(Un, pr, cflR, to_work<R>(dx));
-                my_dt = umin64(my_dt, dbits(cand));
+                if constexpr (sizeof(R) == 8) {
+                    if (!cfl_above(Un, pr, cflR, dx, best_dt)) {
+                        const double cand = cfl_candidate<R>(Un, pr, cflR, dx);
+                        my_dt = umin64(my_dt, dbits(cand));
+                        const float cf = d2f_bits(cand);
+                        if (cf > 0.0f && cf < best_dt) best_dt = cf;
+                    }
+                } else {
+                    const double cand = cfl_candidate<R>(Un, pr, cflR, to_work<R>(dx));
+                    my_dt = umin64(my_dt, dbits(cand));
+                }
             }
         }
         if (a.tile_inst) {
             flush_dt(dtn, my_dt);            // boxes have their own time steps
             my_dt = ~0ull;
+            best_dt = __int_as_float(0x7F800000);
         }
 
         // ---- restriction of father cells whose eight children are final here: one thread per
