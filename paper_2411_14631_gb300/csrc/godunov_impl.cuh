@@ -206,6 +206,13 @@ struct Smem {
     uint8_t gfull[G::NFULL];
     uint16_t gedge[2 * G::NEDGE];
     std::conditional_t<(G::NP < 256), uint8_t, uint16_t> plist[G::NPN];
+    // FP64 depth-1 tiles of a tree: which predicted cells are updated and which refined (bits), and
+    // the faces and predicted cells the update needs
+    static constexpr bool LISTS = sizeof(R) == 8 && D == 1 && RS != AMR_RIEMANN_MLP;
+    static constexpr int NW = LISTS ? (G::NP + 31) / 32 : 1;
+    uint32_t upd[NW], refd[NW];
+    int32_t count[2];
+    uint8_t flist[LISTS ? 3 * G::NF : 1], nlist[LISTS ? G::NPN : 1];
     uint8_t outside[3];             // per tile (index modulo 3): whether a slot lies beyond an outflow face
 };
 static_assert(Geo<2>::NSLOT <= 256, "slot indices fit a byte");
@@ -229,18 +236,25 @@ template <int D> __device__ __forceinline__ TileFace tile_face(int f)
     return t;
 }
 
+// the predicted cell (index) on the left of a face
+template <int D> __device__ __forceinline__ int face_cell(const TileFace &t)
+{
+    using G = Geo<D>;
+    const int fa = t.r0 % (G::CI + 1), t1 = (t.r0 / (G::CI + 1)) % G::CI, t2 = t.r0 / ((G::CI + 1) * G::CI);
+    // predicted-cell coordinates (stencil - 1)
+    const int Lx = t.d == 0 ? fa : 1 + t1;
+    const int Ly = t.d == 0 ? 1 + t1 : t.d == 1 ? fa : 1 + t2;
+    const int Lz = t.d == 2 ? fa : 1 + t2;
+    return Lx + G::P * (Ly + G::P * Lz);
+}
+
 // left and right states of a face (face-normal frame), floored
 template <typename R, int D, int RS>
 __device__ __forceinline__ void face_states(const Smem<R, D, RS> &sm, const TileFace &t, const Prm<R> &pr, R WL[NV],
                                             R WR[NV])
 {
     using G = Geo<D>;
-    const int fa = t.r0 % (G::CI + 1), t1 = (t.r0 / (G::CI + 1)) % G::CI, t2 = t.r0 / ((G::CI + 1) * G::CI);
-    // predicted-cell coordinates (stencil - 1) of the left cell
-    const int Lx = t.d == 0 ? fa : 1 + t1;
-    const int Ly = t.d == 0 ? 1 + t1 : t.d == 1 ? fa : 1 + t2;
-    const int Lz = t.d == 2 ? fa : 1 + t2;
-    const int pl = Lx + G::P * (Ly + G::P * Lz);
+    const int pl = face_cell<D>(t);
     const int pR = pl + (t.d == 0 ? 1 : t.d == 1 ? G::P : G::P * G::P);
     const R *q = &sm.Q[0][0], *dq = &sm.Q[NV + NV * t.d][0];
     const int row[NV] = {0, t.N0 * G::NP, t.T1 * G::NP, t.T2 * G::NP, 4 * G::NP};
@@ -535,6 +549,71 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
             continue;
         }
 
+        // ---- FP64: the faces between an updated cell and one that is not refined, and the
+        // predicted cells beside them.  Where octs are missing or refined that is some two thirds
+        // of a tile's 240 faces and 160 cells, each of which costs the FP64 pipe 61 and 61
+        // operations; the lists cost about 150 integer instructions a warp (in the FP32 kernel
+        // more than they save).
+        using SM = Smem<R, D, RS>;
+        int nface = 3 * G::NF, npred = G::NPN;
+        const bool lists = SM::LISTS && !a.tile_inst && !a.harvest;
+        if constexpr (SM::LISTS) {
+            if (lists) {
+                if (tid < 2) sm.count[tid] = 0;
+                for (int p = tid; p < SM::NW * 32; p += blockDim.x) {
+                    const int i = p % G::P, j = (p / G::P) % G::P, k = p / (G::P * G::P);   // stencil - 1
+                    bool up = false, re = false;
+                    if (p < G::NP) {
+                        const int sl = ((i + 1) >> 1) + G::NS * (((j + 1) >> 1) + G::NS * ((k + 1) >> 1));
+                        const int c = ((i + 1) & 1) + 2 * ((j + 1) & 1) + 4 * ((k + 1) & 1);
+                        re = sm.slot[sl] >= 0 && ((sm.ref[sl] >> c) & 1);
+                        up = sm.slot[sl] >= 0 && !re && i > 0 && i < G::P - 1 && j > 0 && j < G::P - 1 && k > 0 &&
+                             k < G::P - 1;
+                    }
+                    const uint32_t bu = __ballot_sync(0xffffffffu, up), br = __ballot_sync(0xffffffffu, re);
+                    if ((tid & 31) == 0) {
+                        sm.upd[p >> 5] = bu;
+                        sm.refd[p >> 5] = br;
+                    }
+                }
+                __syncthreads();
+                auto bit = [](const uint32_t *w, int p) { return (w[p >> 5] >> (p & 31)) & 1u; };
+                auto used = [&](int p, int q) {      // the face between predicted cells p and q
+                    return ((bit(sm.upd, p) & ~bit(sm.refd, q)) | (bit(sm.upd, q) & ~bit(sm.refd, p))) & 1u;
+                };
+                auto append = [&](bool want, int v, int *count, uint8_t *list) {
+                    const unsigned m = __ballot_sync(0xffffffffu, want);
+                    int base = 0;
+                    if ((tid & 31) == 0 && m) base = atomicAdd(count, __popc(m));
+                    base = __shfl_sync(0xffffffffu, base, 0);
+                    if (want) list[base + __popc(m & ((1u << (tid & 31)) - 1u))] = uint8_t(v);
+                };
+                for (int f0 = 0; f0 < 3 * G::NF; f0 += blockDim.x) {
+                    const int f = f0 + tid;
+                    bool want = false;
+                    if (f < 3 * G::NF) {
+                        const TileFace t = tile_face<D>(f);
+                        const int pl = face_cell<D>(t);
+                        want = used(pl, pl + (t.d == 0 ? 1 : t.d == 1 ? G::P : G::P * G::P));
+                    }
+                    append(want, f, &sm.count[0], sm.flist);
+                }
+                for (int k0 = 0; k0 < G::NPN; k0 += blockDim.x) {
+                    bool want = false;
+                    int p = 0;
+                    if (k0 + tid < G::NPN) {
+                        p = sm.plist[k0 + tid];
+                        const int i = p % G::P, j = (p / G::P) % G::P, k = p / (G::P * G::P);
+                        want = (i > 0 && used(p, p - 1)) || (i < G::P - 1 && used(p, p + 1)) ||
+                               (j > 0 && used(p, p - G::P)) || (j < G::P - 1 && used(p, p + G::P)) ||
+                               (k > 0 && used(p, p - G::P * G::P)) || (k < G::P - 1 && used(p, p + G::P * G::P));
+                    }
+                    append(want, p, &sm.count[1], sm.nlist);
+                }
+                // (the gather's barrier makes the lists visible)
+            }
+        }
+
         // ---- phase 1: gather + primitives of the listed cells (c fastest so a warp reads
         // whole octs)
         for (int kg = tid; kg < G::NG; kg += blockDim.x) {
@@ -594,8 +673,12 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
         // ---- phase 2: slopes + predictor on the listed cells of stencil 1..C-2
         const R lamR = to_work<R>(lam);
         const R hl = R(0.5) * lamR;
-        for (int kp = tid; kp < G::NPN; kp += blockDim.x) {
-            const int p = sm.plist[kp];
+        if (lists) {
+            nface = sm.count[0];
+            npred = sm.count[1];
+        }
+        for (int kp = tid; kp < npred; kp += blockDim.x) {
+            const int p = SM::LISTS && lists ? sm.nlist[kp] : sm.plist[kp];
             const int i = 1 + p % G::P, j = 1 + (p / G::P) % G::P, k = 1 + p / (G::P * G::P);
             const int si = i + G::C * (j + G::C * k);
             const int st[3] = {1, G::C, G::C * G::C};
@@ -661,8 +744,8 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
         if constexpr (RS == AMR_RIEMANN_MLP) {
             mlp_faces<R, D, RS>(sm, sF, pr, a, n_acc, n_fb, n_it, n_solve);
         } else {
-            for (int f = tid; f < 3 * G::NF; f += blockDim.x)
-                face_flux<R, D, RS>(sm, sF, f, pr, a.status, a, t, n_it, n_solve);
+            for (int f = tid; f < nface; f += blockDim.x)
+                face_flux<R, D, RS>(sm, sF, SM::LISTS && lists ? sm.flist[f] : f, pr, a.status, a, t, n_it, n_solve);
         }
         __syncthreads();
         if (a.harvest) continue;   // harvesting only: no update (the loop ends with no barrier due)
