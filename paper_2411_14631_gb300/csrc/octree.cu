@@ -75,7 +75,7 @@ static WsLayout ws_layout(int64_t n)
     W.lxyz = put(16 * n); W.sk0 = put(8 * n); W.sk1 = put(8 * n); W.id0 = put(4 * n); W.id1 = put(4 * n);
     W.flag = put(4 * (n + 1)); W.pos = put(4 * (n + 1));
     W.gflag = put(4 * (8 * n + 1)); W.gpos = put(4 * (8 * n + 1));   // ghost fathers, per cell
-    W.small = put(2048);   // err, tile counts, level histogram, ghost offsets
+    W.small = put(2048);   // err, tile counts, level histogram, reflux offsets, ghost offsets
     W.cub_bytes = cub_bytes_needed(n);
     W.cub = put(W.cub_bytes);
     W.total = o;
@@ -834,13 +834,12 @@ static amr_status build_tree(const amr_geom *geom, const int32_t *h_lxyz, const 
         k_reflux_compact<<<unsigned((c1 - c0 + TB - 1) / TB), TB, 0, st>>>(c0, c1, rflag, rpos, out->reflux_cell);
         k_ghost_bounds<<<1, 32, 0, st>>>(bv, rpos, roff);
         AMR_CUDA_TRY(cudaMemcpyAsync(out->reflux_off, roff, sizeof(out->reflux_off), cudaMemcpyDeviceToHost, st));
-        AMR_CUDA_TRY(cudaStreamSynchronize(st));
     }
     // ghost fathers: one index per coarse leaf the tiles interpolate from, in cell order
     {
         const int64_t ncell = 8 * n;
         int32_t *gflag = (int32_t *)(S + W.gflag), *gpos = (int32_t *)(S + W.gpos);
-        int64_t *goff = (int64_t *)(S + W.small + 1280);
+        int64_t *goff = (int64_t *)(S + W.small + 1536);
         out->ghost_cell = (int32_t *)(T + L.ghost);
         AMR_CUDA_TRY(cudaMemsetAsync(gflag, 0, 4 * size_t(ncell + 1), st));
         for (int d = 0; d < 2; ++d) {
