@@ -794,8 +794,9 @@ def study_poisson(args):
     # FP64 pipe: 1.25 TFLOP/s nominal = 0.625e12 DFMA/s, i.e. 2 DP instructions per clock
     # per SM at 2.07 GHz on 152 SMs
     fp64_peak = 152 * 2 * 2.07e9
-    # algorithmic DP instructions and HBM bytes per cell and iteration
-    alg = {abi.PRECOND_IP: (23, 16 * 8), abi.PRECOND_NONE: (14, 12 * 8)}
+    # algorithmic DP instructions and HBM bytes per cell and iteration (with the preconditioner
+    # the single-reduction form, six vectors read and written; without it the pipelined one)
+    alg = {abi.PRECOND_IP: (18, 12 * 8), abi.PRECOND_NONE: (14, 12 * 8)}
     out = {"study": "Poisson solve on a %d^3 Dirichlet box, CG vs PPCG (Sec. 2.3, Fig. 4)" % N,
            "data": "synthetic: 64 Plummer clumps (core 0.005, contrast 1e4, truncated at r = 0.1), "
                    "b = -4 pi h^2 (rho - mean)", "cells": n, "tol": 1e-4,

@@ -22,15 +22,16 @@
 // sum x-left, x-right, y-left, y-right, z-below, z-above, FP64 update, CFL candidate,
 // restriction), so the states are bitwise those of the other kernels.
 //
-// Bound: latency and issue, not bandwidth (0.9 ms for 1.34 GB of algorithmic traffic at 256^3;
-// issue 50% active, 31.2 warp instructions per update, 24 warps per SM at 80 registers).  A
+// Bound: latency and issue, not bandwidth (0.83 ms for 1.34 GB of algorithmic traffic at 256^3;
+// issue 52% active, 31.2 warp instructions per update, 24 warps per SM at 80 registers).  A
 // single role of 256 threads needed 128 registers (the gather's FP64 loads live across the
 // predictor): 16 warps per SM, 37.9 warp instructions per update.  256^3 step on a GB300: 1.137
 // ms with one role; 1.03 with the roles; 0.97 with look-ups a plane ahead of their use and the
 // L2 prefetch; 0.93 without a branch in the Riemann solver; 0.91 with the range clamps of the
 // conversions in one instruction and the CFL step from the largest signal speed; 0.88 with the
-// restriction first in its warps' iteration.  Without the gather's loads it would take 0.80,
-// without restriction 0.80, without Uo's loads 0.85, without x and y faces 0.86.
+// restriction first in its warps' iteration (0.866 with the restriction launches below it by
+// variable).  At 0.91, without the gather's loads it would take 0.80, without restriction 0.80,
+// without the old states' loads 0.85, without x and y faces 0.86.
 #pragma once
 #include <type_traits>
 #include "godunov_col.cuh"
