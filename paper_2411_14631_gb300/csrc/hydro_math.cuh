@@ -466,24 +466,26 @@ __device__ __forceinline__ double cfl_candidate(const double U[NV], const Prm<R>
 // FP64: whether the candidate of a cell is surely above best_dt, so that it need not be formed
 // (22 FP64 operations of some 480 a cell; one to two cells in ten need it).  From an FP32 estimate
 // of the cell's signal speed, on the FP32 and integer pipes, which the FP64 kernels leave idle.
-// Its error: with the internal energy at least 1e-5 of the total, c^2 loses at most 5% to
-// cancellation where c is smallest against |u|, under 0.2% of the signal speed for gamma (gamma -
-// 1) <= 25; the 2% kept in hand cover that and the roundings.  False (form the candidate) outside
-// these conditions, near the floors, and for anything not finite.
+// Its error: gamma - 1 is formed in FP64 (in FP32 its rounding alone would be 6e-8 / (gamma - 1) of
+// it) and gamma (gamma - 1) e stays a normal FP32 number, so that any gamma above 1 will do; with
+// the internal energy at least 1e-5 of the total, c^2 loses at most 5% to cancellation where c is
+// smallest against |u|, under 0.2% of the signal speed for gamma (gamma - 1) <= 25; the 2% kept in
+// hand cover that and the roundings.  False (form the candidate) outside these conditions, near the
+// floors, and for anything not finite.
 __device__ __forceinline__ bool cfl_above(const double U[NV], const Prm<double> &p, double cfl, double dx, float best_dt)
 {
     if (!(best_dt < 1e30f)) return false;         // none yet
-    const float g = float(p.gamma), gg = g * (g - 1.0f), num = float(cfl) * float(dx);
+    const float g1 = float(p.gamma - 1.0), gg = float(p.gamma) * g1, num = float(cfl) * float(dx);
     const float r = d2f_bits(U[0]), E = d2f_bits(U[4]);
     float ir, c;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ir) : "f"(r));
     const float u = d2f_bits(U[1]) * ir, v = d2f_bits(U[2]) * ir, w = d2f_bits(U[3]) * ir, Es = E * ir;
-    const float es = Es - 0.5f * (u * u + v * v + w * w);
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(gg * es));
+    const float es = Es - 0.5f * (u * u + v * v + w * w), c2 = gg * es;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(c) : "f"(c2));
     const float sig = (fabsf(u) + fabsf(v)) + (fabsf(w) + 3.0f * c);
     const bool ok = gg <= 25.0f && r >= 1e-30f && r <= 1e30f && r > 1.01f * float(p.rho_floor) && Es <= 1e30f &&
-                    Es >= 1e-30f && es > 1e-5f * Es && (g - 1.0f) * es * r > 1.01f * float(p.p_floor) && num >= 1e-30f &&
-                    num <= 1e30f && best_dt >= 1e-30f;
+                    Es >= 1e-30f && es > 1e-5f * Es && c2 >= 1e-36f && g1 * es * r > 1.01f * float(p.p_floor) &&
+                    num >= 1e-30f && num <= 1e30f && best_dt >= 1e-30f;
     return ok && num > best_dt * (sig * 1.02f);
 }
 
