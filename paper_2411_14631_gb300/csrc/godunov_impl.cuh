@@ -183,8 +183,9 @@ __device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsig
 
 // threads per CTA: depth-1 tiles (512 stencil cells) 128, depth-2 tiles (1728) 512.  A
 // depth-2 CTA's shared memory admits one per SM, so it may take every register (no
-// spills); the FP32 depth-1 update (HLLC or exact) fits 64 registers, eight CTAs per SM;
-// the FP64 and surrogate variants keep the compiler's own budget.
+// spills); the FP32 depth-1 update (HLLC or exact) fits 64 registers, eight CTAs per SM; the FP64
+// HLLC update takes what three CTAs per SM leave it; the FP64 exact solver and the surrogate
+// variants keep the compiler's own budget.
 template <int D> __host__ __device__ constexpr int threads_for() { return D == 1 ? 128 : 512; }
 template <typename R, int D, int RS> constexpr int min_ctas_for()
 {
@@ -206,9 +207,10 @@ struct Smem {
     uint8_t gfull[G::NFULL];
     uint16_t gedge[2 * G::NEDGE];
     std::conditional_t<(G::NP < 256), uint8_t, uint16_t> plist[G::NPN];
-    // FP64 depth-1 tiles of a tree: which predicted cells are updated and which refined (bits), and
-    // the faces and predicted cells the update needs
-    static constexpr bool LISTS = sizeof(R) == 8 && D == 1 && RS != AMR_RIEMANN_MLP;
+    // FP64 depth-1 tiles of a tree, HLLC: which predicted cells are updated and which refined (bits),
+    // and the faces and predicted cells the update needs.  (The exact solver and the surrogate report
+    // what they met at every face, in d_status and d_counters, and leave none out.)
+    static constexpr bool LISTS = sizeof(R) == 8 && D == 1 && RS == AMR_RIEMANN_HLLC;
     static constexpr int NW = LISTS ? (G::NP + 31) / 32 : 1;
     uint32_t upd[NW], refd[NW];
     int32_t count[2];
@@ -543,8 +545,8 @@ __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) 
         have_nx = t_nx < a.t_end;
         if (have_nx && tid < G::NSLOT) e_nx = a.tile_slot[t_nx * G::NSLOT + tid];
         // every cell refined (the middle of a finer level): nothing of this tile is updated, and
-        // no face of it is used
-        if (!any_updated && !a.harvest) {
+        // no face of it is used (HLLC: no face reports anything either)
+        if (RS == AMR_RIEMANN_HLLC && !any_updated && !a.harvest) {
             if (have_nx && tid < G::NSLOT) rf_nx = e_nx >= 0 ? tv.refmask[e_nx] : 0;
             continue;
         }
