@@ -4,72 +4,12 @@
 #include <cmath>
 #include <cuda_runtime.h>
 #include "../../include/amrhydro.h"
+#include "launch.cuh"
 
 namespace amr {
 
 constexpr int NV = 5;
 constexpr int32_t OUTSIDE = INT32_MIN;   // nb27 / slot entry beyond an outflow face
-
-#define AMR_CUDA_TRY(expr)                                  \
-    do {                                                    \
-        cudaError_t e_ = (expr);                            \
-        if (e_ != cudaSuccess) return AMR_ECUDA;            \
-    } while (0)
-
-// Launch of a kernel that needs `smem` bytes of dynamic shared memory: how many of its CTAs are
-// resident on the GPU at once, and its attributes set.  Both are properties of (kernel, device)
-// and are looked up once per host thread: the three calls take some 20 us of host time, more
-// than a small level's kernel.  After cudaDeviceReset the attributes are gone and a launch
-// fails with cudaErrorInvalidValue: launch_kernel then sets them again and repeats it.
-struct LaunchCache {
-    struct Entry {
-        const void *kern;
-        int dev, resident;
-    };
-    Entry e[64];
-    int n = 0;
-};
-inline LaunchCache &launch_cache()
-{
-    thread_local LaunchCache c;
-    return c;
-}
-inline amr_status launch_setup(const void *kern, int threads, size_t smem, bool all_smem, int *resident)
-{
-    LaunchCache &c = launch_cache();
-    int dev = 0, nsm = 0, per_sm = 0;
-    AMR_CUDA_TRY(cudaGetDevice(&dev));
-    for (int i = 0; i < c.n; ++i)
-        if (c.e[i].kern == kern && c.e[i].dev == dev) {
-            *resident = c.e[i].resident;
-            return AMR_OK;
-        }
-    AMR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    if (all_smem) AMR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
-    AMR_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    *resident = per_sm * nsm;
-    if (c.n < 64) c.e[c.n++] = {kern, dev, *resident};
-    return AMR_OK;
-}
-// kern<<<grid(resident), threads, smem>>>(arg), grid computed from the resident CTAs
-template <typename A, typename G>
-inline amr_status launch_kernel(void (*kern)(A), int threads, size_t smem, bool all_smem, cudaStream_t st, A &arg,
-                                G grid)
-{
-    for (int attempt = 0;; ++attempt) {
-        int resident = 0;
-        const amr_status r = launch_setup(reinterpret_cast<const void *>(kern), threads, smem, all_smem, &resident);
-        if (r != AMR_OK) return r;
-        const unsigned nb = grid(int64_t(resident), arg);
-        kern<<<nb, threads, smem, st>>>(arg);
-        const cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess) return AMR_OK;
-        if (e != cudaErrorInvalidValue || attempt) return AMR_ECUDA;
-        launch_cache().n = 0;
-    }
-}
 
 // First error wins; 0 means no error.
 __device__ __forceinline__ void set_error(int32_t *word, int32_t code)
