@@ -459,8 +459,9 @@ amr_status hydro_conservation(const amr_tree *tree, const double *d_u, double *d
    against IEEE conversions; the paper has no counterpart (its code is FP64 throughout).
    hydro_state_to_fp32: d_y[i] = the FP32 value the FP32 path reads for the FP64 state
    value d_x[i]: round to nearest, ties away from zero (IEEE rounds ties to even); |x|
-   below 2^-126 gives a signed zero; |x| >= 2^128, +-Inf and NaN give a non-finite float
-   of the same sign (+-Inf or a NaN).  hydro_state_from_fp32: d_x[i] = the FP64 value of
+   below 2^-126 gives a signed zero (where it rounds to 2^-126, that is from 2^-126 (1 -
+   2^-25) up, the update kernels read 2^-126); |x| >= 2^128, +-Inf and NaN give a
+   non-finite float of the same sign (+-Inf or a NaN).  hydro_state_from_fp32: d_x[i] = the FP64 value of
    the FP32 value d_y[i] (exact; +-Inf and NaN kept; FP32 denormals give a signed zero).
    Device arrays of n >= 0 elements; AMR_EINVAL for n < 0 or a NULL array with n > 0;
    asynchronous on the stream. */

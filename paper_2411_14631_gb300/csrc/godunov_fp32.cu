@@ -1,6 +1,7 @@
 // FP32 instantiation of the tiled Godunov kernel: reconstruction, predictor and Riemann
 // solve in FP32 (compiled with fast single-precision division and square root), state
 // accumulation in FP64.
+#define AMR_FLUSHES_DENORMALS
 #include "godunov_impl.cuh"
 
 namespace amr {

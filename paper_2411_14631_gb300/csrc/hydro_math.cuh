@@ -33,9 +33,10 @@ __device__ __forceinline__ float d2f_bits(double x)
     return __uint_as_float(m | (hi & 0x80000000u));
 }
 
-// The same where denormal values are flushed by their use (the FP32 kernels), both ends of the
-// range clamped by one instruction: 6 integer operations instead of 8.  Where d2f_bits gives
-// a zero for |x| < 2^-126 this gives a denormal (or, rounded up to it, 2^-126).
+// The same for kernels that flush denormals (AMR_FLUSHES_DENORMALS), both ends of the range clamped by
+// one instruction: 6 integer operations instead of 8.  Below 2^-126 this gives denormal patterns of
+// no use except to be flushed; from 2^-126 (1 - 2^-25) up it rounds to 2^-126, where d2f_bits gives
+// zero.
 __device__ __forceinline__ float d2f_ftz(double x)
 {
     const unsigned hi = unsigned(__double2hiint(x)), lo = unsigned(__double2loint(x));
@@ -84,10 +85,15 @@ template <> __device__ __forceinline__ bool state_finite<float>(const double U[5
     return fabsf(s) <= 3.402823466e38f;
 }
 
-// working-precision view of an FP64 state value, and back
+// working-precision view of an FP64 state value, and back.  godunov_fp32.cu, whose kernels flush
+// denormals (--use_fast_math), defines AMR_FLUSHES_DENORMALS; elsewhere a denormal would be used.
 template <typename R> __device__ __forceinline__ R to_work(double x);
 template <> __device__ __forceinline__ double to_work<double>(double x) { return x; }
+#ifdef AMR_FLUSHES_DENORMALS
 template <> __device__ __forceinline__ float to_work<float>(double x) { return d2f_ftz(x); }
+#else
+template <> __device__ __forceinline__ float to_work<float>(double x) { return d2f_bits(x); }
+#endif
 __device__ __forceinline__ double to_state(double x) { return x; }
 __device__ __forceinline__ double to_state(float x) { return f2d_bits(x); }
 
