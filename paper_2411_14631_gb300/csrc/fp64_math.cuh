@@ -7,12 +7,13 @@
 //   - reciprocal and division start from the hardware's approximations (rcp.approx.ftz.f64,
 //     rsqrt.approx.ftz.f64, off the FP64 pipe) and take one third-order step (Householder;
 //     Markstein 2000, "IA-64 and Elementary Functions", for the division's exact remainder):
-//     3 operations for a reciprocal, 6 for a division, with IEEE's result (in a restatement
-//     in C with seeds 2^-20 off, 0.507 ulp at most, and all of 3 million divisions equal);
+//     3 operations for a reciprocal, 6 for a division.  Against 113-bit arithmetic, 8 million random
+//     operands: the reciprocal within 0.506 ulp (0.03% differ from IEEE's, by one unit), every
+//     division IEEE's;
 //   - the sound speed sqrt(a / r) is one reciprocal square root of a r, 8 operations, within
-//     1.0 ulp (a rounded square root of a rounded quotient: 0.85 ulp);
+//     1.0 ulp, rms 0.328 (a rounded square root of a rounded quotient: 0.85, rms 0.326);
 //   - comparisons and MinMod are integer operations on the bit patterns, with the same
-//     results, also for zeros, infinities and NaN.
+//     results, also for zeros (a zero MinMod up to its sign), infinities and NaN.
 // Operands out of the middle of the exponent range take the IEEE operations (one function
 // each, not inlined).
 #pragma once
@@ -91,8 +92,8 @@ __device__ __forceinline__ double floor_at(double a, double f)
     return ia - jf - 1ull < 0x7FF0000000000000ull - jf ? a : f;
 }
 
-// MinMod of two differences (results of subtractions): zero when their signs differ, else the
-// one of smaller magnitude; the other one when one is NaN.  The median (0, a, b) of
+// MinMod of two differences (results of subtractions): zero when their signs differ or both are NaN,
+// else the one of smaller magnitude; the other one when one is NaN.  The median (0, a, b) of
 // fmin / fmax, bit for bit up to the sign of a zero.
 __device__ __forceinline__ double minmod64(double a, double b)
 {
@@ -101,8 +102,9 @@ __device__ __forceinline__ double minmod64(double a, double b)
     const unsigned long long ma = (unsigned long long)ia & top, mb = (unsigned long long)ib & top;
     const long long r = ma < mb ? ia : ib;
     const bool opposite = int(unsigned(ia >> 32) ^ unsigned(ib >> 32)) < 0;
-    const bool finite = max(unsigned(ma >> 32), unsigned(mb >> 32)) <= 0x7FF00000u;
-    return opposite && finite ? 0.0 : __longlong_as_double(r);
+    const unsigned ha = unsigned(ma >> 32), hb = unsigned(mb >> 32);
+    const bool none_nan = max(ha, hb) <= 0x7FF00000u, both_nan = min(ha, hb) > 0x7FF00000u;
+    return (opposite && none_nan) || both_nan ? 0.0 : __longlong_as_double(r);
 }
 
 }  // namespace amr
