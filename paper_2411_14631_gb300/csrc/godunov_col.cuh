@@ -59,9 +59,10 @@ struct ColArgs {
     const int64_t *inst_col_off, *inst_oct_off;
     // the z planes of every column, column after column (box after box): CTA i takes planes
     // [i share, (i + 1) share), a segment per column it meets; with zc > 0 no segment is
-    // longer than zc and each CTA takes one (share = zc, columns padded to multiples of zc)
-    int64_t planes, share;
-    int zc;
+    // longer than zc and each CTA takes one (share = zc, columns padded to multiples of zc).
+    // Where an equal share would be longer than share_max, zc becomes long_zc.
+    int64_t planes, share, share_max;
+    int zc, long_zc;
     int32_t finer;          // the level has refined cells (finer levels exist)
     int level;
     int64_t n;              // cells per dimension
@@ -529,6 +530,7 @@ __global__ void __launch_bounds__(256) k_godunov_col(ColArgs a)
 // grid of a z-column kernel: equal shares, one per resident CTA, or segments of a.zc planes
 inline unsigned column_grid(int64_t resident, ColArgs &a)
 {
+    if (a.zc == 0 && even_share(a.planes, resident) > a.share_max) a.zc = a.long_zc;
     a.share = a.zc > 0 ? a.zc : even_share(a.planes, resident);
     return unsigned((a.planes + a.share - 1) / a.share);
 }
@@ -546,6 +548,13 @@ amr_status launch_col(const amr_tree *t, const hydro_params *p, const double *u_
     a.inst_oct_off = t->inst_oct_off;
     a.finer = t->n_inst == 0 && t->grid_level < t->levelmax;
     a.zc = 0;
+    // FP32: equal shares only up to a column's height, in a batch half the smallest box's.  Longer
+    // ones leave neighbouring columns at different heights, whose halos then come from memory, and
+    // cut short columns in two: 256^3 1165 us with segments of 64 planes, 1246 with shares of 430;
+    // 100 boxes of 16^3 56 / 61, 256 of them 99 / 106, 300 of 32^3 687 / 715; but 128^3 205 / 193, 64^3
+    // 71 / 56, 64 boxes of 16^3 48 / 43.  The FP64 kernel, bound by its pipe, takes them always.
+    a.share_max = sizeof(R) == 8 ? INT64_MAX : t->n_inst > 0 ? 8 : int64_t(1) << t->grid_level;
+    a.long_zc = t->n_inst > 0 ? 16 : t->grid_level < 6 ? 1 << t->grid_level : 64;
     if (t->n_inst > 0) {
         a.level = 0;
         a.n = 0;

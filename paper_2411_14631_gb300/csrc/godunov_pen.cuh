@@ -475,7 +475,8 @@ amr_status launch_pen(const amr_tree *t, const hydro_params *p, const double *u_
     a.inst_col_off = t->inst_col_off;
     a.inst_oct_off = t->inst_oct_off;
     a.finer = t->n_inst == 0 && t->grid_level < t->levelmax;
-    a.zc = 0;
+    a.zc = a.long_zc = 0;
+    a.share_max = INT64_MAX;
     if (t->n_inst > 0) {
         if (t->col_work <= 0 || t->col_work % 4) return AMR_EINVAL;
         a.level = 0;
