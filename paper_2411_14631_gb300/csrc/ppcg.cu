@@ -645,7 +645,9 @@ amr_status plan(const ppcg_params *prm, Launch &L)
     L.ty = prm->tile_y ? prm->tile_y : L.pipe ? 8 : 16;
     const int cy = (ny + L.ty - 1) / L.ty;
     const int64_t cols = (int64_t)cx * cy;
-    if (cy > 65535 || (seg > 0 && (nz + seg - 1) / seg > 65535)) return AMR_EINVAL;
+    // (the limit of rows is that of the tile height that a caller who leaves it open may rely on)
+    const int limit_ty = prm->tile_y ? prm->tile_y : 8;
+    if ((ny + limit_ty - 1) / limit_ty > 65535 || (seg > 0 && (nz + seg - 1) / seg > 65535)) return AMR_EINVAL;
     if (L.pipe) {
         if (seg == 0) {
             int64_t nseg = (INIT_BLOCKS + cols - 1) / cols;
