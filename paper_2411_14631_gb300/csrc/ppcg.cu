@@ -626,12 +626,60 @@ struct Launch {
     March mc;
 };
 
-// Which kernel, tile height and split of the z planes.  Single-reduction form: with the
-// preconditioner, on boxes of at least SINGLE_CELLS cells.  Per iteration, pipelined against
-// single-reduction: 64^3 30.9 / 32.8 us, 180 x 141 x 117 187 / 164, 256^3 825 / 740; without
-// preconditioner the forms take the same FP64 work, and the pipelined one needs one halo instead
-// of three: 64^3 20.9 / 22.6, 256^3 483 / 472.
+// Which kernel.  Single-reduction form: with the preconditioner, on boxes of at least SINGLE_CELLS
+// cells and SINGLE_PLANES planes (below, the planes its halo adds on either side cost more than its
+// recurrences save: 800 x 300 x 3 56 us an iteration against 60).  Per iteration, pipelined against
+// single-reduction: 64^3 30.9 / 32.8 us, 180 x 141 x 117 187 / 164, 256^3 826 / 717, flat and narrow boxes
+// at single_split; without preconditioner the forms take the same FP64 work, and the pipelined one
+// needs one halo instead of three: 64^3 20.9 / 22.6, 256^3 483 / 472.
 constexpr int64_t SINGLE_CELLS = 700000;
+constexpr int SINGLE_PLANES = 5;
+
+// Tile height and split of the planes for the single-reduction form: the ones with the shortest
+// estimated time, in plane steps of an SM that holds every block it can (6.4 us).  A block's planes
+// cost it three more for the halo.  Segments of one length run in waves; in one that leaves the
+// SMs with fewer blocks a plane step is shorter (BUSY, by the blocks of the fullest SM, measured).
+// Equal shares of all planes, in one wave, pay the halo once more per column that a block goes on
+// to, about 2.5 planes, and read more of it from memory (3.5%; neighbouring columns are at
+// different heights): they repay it where whole waves of segments do not come out even.  16 rows
+// repeat less of the halo, 8 waste fewer rows of a low box.  us an iteration, pipelined against this
+// choice: 300 x 300 x 9 72 / 64, 300 x 300 x 16 101 / 92, 190 x 33 x 190 91 / 88, 16 x 16 x 3000 97 / 83,
+// 24 x 24 x 1300 75 / 68, 9 x 9 x 9000 187 / 122, 1 x 1 x 800000 2080 / 1440; over 140 boxes of 0.7 to 17 M
+// cells 0.89 in the mean, none slower.  (Segments, at most 64 of them, where a last wave was not half
+// empty, and always 16 rows: 74, 108, 99, 187, 97, 121 and 2870.)
+constexpr double BUSY8[4] = {0.44, 0.68, 0.89, 1.04}, BUSY16[2] = {0.68, 1.0};
+struct Split {
+    double cost = -1.0;
+    int ty = 0, seg = 0;      // seg 0: equal shares
+    int64_t share = 0;
+    void offer(double c, int y, int s, int64_t sh)
+    {
+        if (cost < 0.0 || c < cost) {
+            cost = c;
+            ty = y;
+            seg = s;
+            share = sh;
+        }
+    }
+};
+void single_split(int nx, int ny, int nz, int ty, int nsm, Split &best)
+{
+    const int per_sm = 1024 / (TX * ty);
+    const double *busy = ty == 8 ? BUSY8 : BUSY16;
+    const int64_t cols = (int64_t)((nx + TX - 1) / TX) * ((ny + ty - 1) / ty), slots = (int64_t)nsm * per_sm;
+    const int64_t most = 4 * slots / cols + 1;                 // segments of a column: four waves at most
+    for (int64_t nseg = 1; nseg <= most && nseg <= nz; nseg++) {
+        int s = (int)((nz + nseg - 1) / nseg);
+        if (s < MIN_SEG) s = MIN_SEG;
+        const int64_t blocks = cols * ((nz + s - 1) / s), rest = blocks % slots;
+        double waves = double(blocks / slots) * busy[per_sm - 1];
+        if (rest) waves += busy[(rest + nsm - 1) / nsm - 1];
+        best.offer(waves * ((s < nz ? s : nz) + 3), ty, s, s);
+    }
+    int64_t share = (cols * nz + slots - 1) / slots;
+    if (share < 2) share = 2;
+    best.offer(1.035 * (double(share) + 2.5 * (1.0 + double(share) / nz)) * busy[per_sm - 1], ty, 0, share);
+}
 
 amr_status plan(const ppcg_params *prm, Launch &L)
 {
@@ -639,17 +687,13 @@ amr_status plan(const ppcg_params *prm, Launch &L)
     int seg = prm->seg;
     if (prm->tile_y != 0 && prm->tile_y != 8 && prm->tile_y != 16) return AMR_EINVAL;
     if (seg != 0 && seg < MIN_SEG) return AMR_EINVAL;
-    L.pipe = prm->precond != PPCG_PRECOND_IP || (int64_t)nx * ny * nz < SINGLE_CELLS;
-    // 16 rows repeat less of the halo in the single-reduction form (20 instead of 22 FP64
-    // operations a cell): 256^3 715 us an iteration against 757, 180 x 141 x 117 164 against 168
-    L.ty = prm->tile_y ? prm->tile_y : L.pipe ? 8 : 16;
+    L.ty = prm->tile_y ? prm->tile_y : 8;
     const int cy = (ny + L.ty - 1) / L.ty;
-    const int64_t cols = (int64_t)cx * cy;
-    // (the limit of rows is that of the tile height that a caller who leaves it open may rely on)
-    const int limit_ty = prm->tile_y ? prm->tile_y : 8;
-    if ((ny + limit_ty - 1) / limit_ty > 65535 || (seg > 0 && (nz + seg - 1) / seg > 65535)) return AMR_EINVAL;
+    if (cy > 65535 || (seg > 0 && (nz + seg - 1) / seg > 65535)) return AMR_EINVAL;
+    L.pipe = prm->precond != PPCG_PRECOND_IP || (int64_t)nx * ny * nz < SINGLE_CELLS || nz < SINGLE_PLANES;
     if (L.pipe) {
         if (seg == 0) {
+            const int64_t cols = (int64_t)cx * cy;
             int64_t nseg = (INIT_BLOCKS + cols - 1) / cols;
             seg = (int)((nz + nseg - 1) / nseg);
             if (seg < MIN_SEG) seg = MIN_SEG;
@@ -660,39 +704,22 @@ amr_status plan(const ppcg_params *prm, Launch &L)
         L.grid = dim3(cx, cy, cz);
         return AMR_OK;
     }
-    int dev = 0, nsm = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t slots = (int64_t)nsm * (1024 / (TX * L.ty));
     L.mc.cx = cx;
-    L.mc.seg = seg;
-    if (seg == 0) {
-        // Segments of one length: the one with the shortest estimated time, whole waves of
-        // resident blocks, each its planes plus about three planes' worth of halo.  Where that
-        // leaves the last wave half empty, equal shares of all planes in one wave instead
-        // (180 x 141 x 117: 164 us an iteration against 170).  Not otherwise: neighbouring columns
-        // are then at different heights and re-read each other's halo from memory.
-        int64_t best = -1;
-        for (int nseg = 1; nseg <= 64 && nseg <= nz; nseg++) {
-            int s = (nz + nseg - 1) / nseg;
-            if (s < MIN_SEG) s = MIN_SEG;
-            const int64_t blocks = cols * ((nz + s - 1) / s);
-            const int64_t cost = ((blocks + slots - 1) / slots) * (s + 3);
-            if (best < 0 || cost < best) {
-                best = cost;
-                L.mc.seg = s;
-            }
-        }
-        const int64_t share = (cols * nz + slots - 1) / slots;
-        if (share >= 12 && double(share) + 2.5 * (1.0 + double(share) / nz) < 0.9 * double(best)) {
-            L.mc.seg = 0;
-            L.mc.share = share;
-            L.mc.planes = cols * nz;
-        }
+    L.mc.seg = L.mc.share = seg;
+    if (seg > 0) {
+        if (!prm->tile_y) L.ty = 16;
+    } else {
+        int dev = 0, nsm = 152;
+        if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        Split best;
+        for (int ty = 16; ty >= 8; ty -= 8)
+            if (!prm->tile_y || prm->tile_y == ty) single_split(nx, ny, nz, ty, nsm, best);
+        L.ty = best.ty;
+        L.mc.seg = best.seg;
+        L.mc.share = best.share;
     }
-    if (L.mc.seg > 0) {
-        L.mc.share = L.mc.seg;
-        L.mc.planes = cols * ((nz + L.mc.seg - 1) / L.mc.seg) * L.mc.seg;
-    }
+    const int64_t cols = (int64_t)cx * ((ny + L.ty - 1) / L.ty);
+    L.mc.planes = L.mc.seg > 0 ? cols * ((nz + L.mc.seg - 1) / L.mc.seg) * L.mc.seg : cols * nz;
     const int64_t blocks = (L.mc.planes + L.mc.share - 1) / L.mc.share;
     if (blocks > INT32_MAX) return AMR_EINVAL;
     L.grid = dim3((unsigned)blocks);
