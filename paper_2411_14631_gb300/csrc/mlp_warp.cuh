@@ -170,10 +170,8 @@ __device__ __forceinline__ void input_frag(const float *x16, int lane, uint32_t 
 }
 
 // Forward pass of 16 samples.  Output: lanes with t == 0 hold y[g] (y0[0], y0[1]) and
-// y[g+8] (y1[0], y1[1]).  If z is given, the pre-activations of the three hidden layers
-// are kept (accumulator layout) for a backward pass.
-__device__ __forceinline__ void forward16(const Packed &P, const float *x16, int lane, float out[4],
-                                          float (*z)[8][4] = nullptr)
+// y[g+8] (y1[0], y1[1]).
+__device__ __forceinline__ void forward16(const Packed &P, const float *x16, int lane, float out[4])
 {
     uint32_t a0[4];
     input_frag(x16, lane, a0);
@@ -188,20 +186,8 @@ __device__ __forceinline__ void forward16(const Packed &P, const float *x16, int
     uint32_t a[4][4];
 #pragma unroll
     for (int layer = 0; layer < 2; ++layer) {
-        if (z) {
-#pragma unroll
-            for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) z[layer][nt][i] = acc[nt][i];
-        }
         acc_to_a_silu(acc, a);
         hidden64(a, P.w + (layer == 0 ? PW2 : PW3), P.b + H * (layer + 1), acc, lane);
-    }
-    if (z) {
-#pragma unroll
-        for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) z[2][nt][i] = acc[nt][i];
     }
     acc_to_a_silu(acc, a);
     const int t = lane & 3;
