@@ -1,5 +1,5 @@
 // FP64 instantiation of the tiled Godunov kernel: every operation of the scheme in FP64
-// (the plain path; IEEE division and square root).
+// (the plain path; divisions and sound speeds by fp64_math.cuh).
 #include "godunov_impl.cuh"
 
 namespace amr {

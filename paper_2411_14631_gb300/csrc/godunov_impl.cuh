@@ -411,8 +411,8 @@ __device__ __forceinline__ void mlp_faces(Smem<R, D, RS> &sm, R (*sF)[NV][Geo<D>
     }
 }
 
-// Riemann problem at face r0 of direction DIR: left state = predicted cell + half its
-// slope, right state = next cell - half its slope (floored), in the face-normal frame.
+// The update of one level's octs (or of all levels'): a CTA loops over tiles; phases per tile: gather,
+// predictor, Riemann problems, update, restriction and flux-register rows.
 template <typename R, int D, int RS>
 __global__ void __launch_bounds__(threads_for<D>(), (min_ctas_for<R, D, RS>())) k_godunov(GArgs a)
 {

@@ -436,12 +436,9 @@ __device__ __forceinline__ void face_state(const R Wt[NV], const R DlD[NV], R ha
     S[4] = rmax(fmar(half, DlD[4], Wt[4]), pr.p_floor);
 }
 
-// dt candidate of one cell: cfl * dx / sum_d (|u_d| + c), from the FP64 state; p, cfl and
-// dx already in the working precision
-// FP32, in two parts: the candidate of a cell falls with its signal speed sum_d (|u_d| + c)
-// (rcp.approx.ftz.f32, which the division is made of, falls monotonically over all normal
-// floats: checked value by value), so the smallest candidate of cells of one size is that
-// of their largest signal speed.
+// The dt candidate of a cell in FP32, in two parts: it falls with the cell's signal speed
+// sum_d (|u_d| + c) (monotonically over all normal floats, tested value by value), so the smallest
+// candidate of cells of one size is that of their largest signal speed.
 __device__ __forceinline__ float cfl_signal(const double U[NV], const Prm<float> &p)
 {
     float W[NV];
@@ -454,6 +451,8 @@ __device__ __forceinline__ double cfl_step(float sig, float cfl, float dx)
     return to_state(cfl * (dx / sig) * 0.9999847412109375f);
 }
 
+// dt candidate of one cell: cfl * dx / sum_d (|u_d| + c), from the FP64 state; p, cfl and
+// dx already in the working precision
 template <typename R>
 __device__ __forceinline__ double cfl_candidate(const double U[NV], const Prm<R> &p, R cfl, R dx)
 {

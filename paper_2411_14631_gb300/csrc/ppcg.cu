@@ -463,10 +463,11 @@ struct March {
     int seg, cx;
 };
 
-// One iteration (see the file comment).  Step k of a block's z march: the residual plane k+2, loaded during the step before, is formed, the loads of the next one and of the own cell's vectors
-// are started, then u of plane k+1 and w of plane k.  The places of a thread's elements in the
-// halo planes are worked out once: doing so per plane and element (two divisions each) took 265
-// integer operations a cell.
+// One iteration (see the file comment).  Step k of a block's z march: the residual plane k+2, loaded
+// during the step before, is formed, the loads of the next one and of the own cell's vectors are
+// started, then u of plane k+1 and w of plane k.  The places of a thread's elements in the halo planes
+// are worked out once: doing so per plane and element (two divisions each) took 265 integer
+// operations a cell.
 template <int TY>
 __global__ void __launch_bounds__(TX *TY, 1024 / (TX * TY)) k_iter(Dims d, Vecs v, double *__restrict__ x, PState *st,
                                                                   double *part, double *eps, March mc)
